@@ -3,6 +3,7 @@
 // Berends-Giele amplitude and the event weight (the four stages of Sec. 3).
 #pragma once
 #include <cstdint>
+#include <type_traits>
 
 #include "tess_bg.cuh"
 #include "tess_math.cuh"
@@ -214,39 +215,48 @@ __device__ __forceinline__ uint32_t sample_config(const EventParams &P, uint64_t
   return hel;
 }
 
-// The same draws as sample_config, with the permutation kept packed: nibble
-// a of the working word holds the leg at colour position a (a swap is a few
-// shifts and xors instead of selects over positions).  Returns the helicity
-// word; *posw receives the inverse, nibble l = colour position of leg l.
+// The same draws as sample_config, with the permutation of legs 1..N-1 over
+// colour positions 1..N-1 (leg 0 stays at position 0) packed in nibbles: one
+// 32-bit word up to N = 9, a 64-bit word above (a swap is a few shifts and
+// xors instead of selects over positions).  Two draws come from each Philox
+// block, and the loop over blocks stays rolled (code size, see kin_ds).
+// Returns the helicity word; *posw receives the inverse, nibble l - 1 =
+// position of leg l, less one (leg_block).
 template <int N>
-__device__ __forceinline__ uint32_t sample_positions(const EventParams &P, uint64_t ev, uint64_t *posw) {
+using PosWord = std::conditional_t<(N <= 9), uint32_t, uint64_t>;
+
+template <int N>
+__device__ __forceinline__ int leg_block(PosWord<N> posw, int l) {
+  return l == 0 ? 0 : (int)((posw >> (4 * (l - 1))) & 15u);
+}
+
+template <int N>
+__device__ __forceinline__ uint32_t sample_positions(const EventParams &P, uint64_t ev, PosWord<N> *posw) {
   static_assert(N <= 16, "4-bit positions");
+  using W = PosWord<N>;
   constexpr int M = N - 2;
-  constexpr uint32_t jh = 2 + 4 * M;  // helicity draw; ordering draws follow
-  uint4 w = event_block(P, ev, jh >> 1);
-  uint32_t cur = jh >> 1;
-  const uint32_t a0 = (jh & 1u) ? w.z : w.x;
-  const uint32_t hel = a0 >> (32 - N);
-  uint64_t pw = 0;
+  constexpr uint32_t jh = 2 + 4 * M;  // helicity draw (even); the M ordering draws follow
+  W pw = 0;
 #pragma unroll
-  for (int a = 0; a < N; ++a) pw |= (uint64_t)a << (4 * a);
-#pragma unroll
-  for (int i = N; i >= 3; --i) {
-    const uint32_t j = jh + 1 + (N - i);
-    if ((j >> 1) != cur) {
-      cur = j >> 1;
-      w = event_block(P, ev, cur);
-    }
-    const uint64_t k = (j & 1u) ? unit_bits(w.z, w.w) : unit_bits(w.x, w.y);
-    const int r = 2 + floor_unit_times(k, (uint32_t)(i - 1));
-    // swap positions i and r (1-based)
-    const int si = 4 * (i - 1), sr = 4 * (r - 1);
-    const uint64_t x = ((pw >> si) ^ (pw >> sr)) & 15ull;
+  for (int a = 0; a < N - 1; ++a) pw |= (W)a << (4 * a);
+  // draw d exchanges position i = N - d (1-based) with 2 + floor(u (i - 1))
+  auto exchange = [&](uint32_t a, uint32_t b, int d) {
+    const int si = 4 * (N - 2 - d), sr = 4 * floor_unit_times(unit_bits(a, b), (uint32_t)(N - 1 - d));
+    const W x = ((pw >> si) ^ (pw >> sr)) & 15u;
     pw ^= (x << si) | (x << sr);
+  };
+  uint4 w = event_block(P, ev, jh >> 1);
+  const uint32_t hel = w.x >> (32 - N);
+  exchange(w.z, w.w, 0);
+#pragma unroll 1
+  for (int d = 1; d < M; d += 2) {
+    w = event_block(P, ev, (jh >> 1) + (uint32_t)(d + 1) / 2);
+    exchange(w.x, w.y, d);
+    if (d + 1 < M) exchange(w.z, w.w, d + 1);
   }
-  uint64_t qw = 0;
+  W qw = 0;
 #pragma unroll
-  for (int a = 0; a < N; ++a) qw |= (uint64_t)a << (4 * (int)((pw >> (4 * a)) & 15ull));
+  for (int a = 0; a < N - 1; ++a) qw |= (W)a << (4 * (int)((pw >> (4 * a)) & 15u));
   *posw = qw;
   return hel;
 }

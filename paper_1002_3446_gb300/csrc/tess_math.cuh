@@ -73,20 +73,16 @@ __device__ __forceinline__ uint64_t unit_bits(uint32_t a, uint32_t b) {
 }
 
 // floor(u * c) exactly as the double-precision product rounds it (single
-// rounding to 53 bits, ties to even), in integer arithmetic: u * c =
-// (2k+1) c 2^-53 and scaling by 2^-53 is exact.  c <= 2^10.
+// rounding to 53 bits, ties to even): u * c = X 2^-53 with X = (2k+1) c < 2^53 c.
+// The rounding moves the floor only when X rounds up to the next multiple of
+// 2^53, from a value whose integer part f has bits_of(f) bits: X is then
+// rounded to 2^bits_of(f), and every bit below 2^53 is set down to the rounding
+// position, so that half a unit (ties included, to even) carries.  c <= 2^10.
 __device__ __forceinline__ int floor_unit_times(uint64_t k, uint32_t c) {
-  uint64_t X = (2 * k + 1) * (uint64_t)c;
-  const int e = 63 - __clzll((long long)X);
-  if (e >= 53) {
-    const int s = e - 52;
-    const uint64_t mask = (1ull << s) - 1, half = 1ull << (s - 1);
-    uint64_t q = X >> s;
-    const uint64_t rem = X & mask;
-    if (rem > half || (rem == half && (q & 1ull))) ++q;
-    X = q << s;
-  }
-  return (int)(X >> 53);
+  const uint64_t X = (2 * k + 1) * (uint64_t)c;
+  const uint32_t f = (uint32_t)(X >> 53);
+  const uint32_t half = (1u << (32 - __clz((int)f))) >> 1;  // f = 0: exact, no rounding
+  return (int)((X + half) >> 53);
 }
 
 // A uniform in single precision from the same two words: hi 2^-26 +

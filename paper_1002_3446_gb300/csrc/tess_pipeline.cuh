@@ -149,43 +149,33 @@ __device__ __forceinline__ void polarisation_angles(const EventParams &P, uint64
   }
 }
 
-// Cuts and observables of the FP32 kinematics forms from the rounded
-// momenta pk (E, px, py, pz of the final-state gluons) and the partonic
-// rapidity y: pT, eta (lab), H_T, leading pT, and the pT / |eta| cuts.
+// Cuts and observables of the FP32 kinematics forms, one final-state gluon:
+// from its rounded momentum pk (E, px, py, pz) and the partonic rapidity y the
+// lab eta, and its part in H_T, the leading pT and the pT / |eta| cuts.
 // Every operation's rounding is written out (no contraction left to the
 // compiler), so the kernels' instantiations (cut-first or not) give
 // bit-identical observables.
-template <int M>
-__device__ __forceinline__ void cuts_observables(const EventParams &P, const float (&pk)[M][4], float y, float (&px)[M],
-                                                 float (&py)[M], float (&pt)[M], float (&eta)[M], int &pass, float &sum,
-                                                 float &lead) {
-#pragma unroll
-  for (int i = 0; i < M; ++i) {
-    px[i] = pk[i][1];
-    py[i] = pk[i][2];
-    const float pz = pk[i][3];
-    const float pt2 = __fmaf_rn(px[i], px[i], __fmul_rn(py[i], py[i]));
-    const float pabs = sqrtf(__fmaf_rn(pz, pz, pt2));
-    pt[i] = sqrtf(pt2);
-    eta[i] = __fadd_rn(__fmul_rn(0.5f, logf(__fdiv_rn(__fadd_rn(pabs, pz), __fsub_rn(pabs, pz)))), y);
-    sum = __fadd_rn(sum, pt[i]);
-    lead = fmaxf(lead, pt[i]);
-    pass &= (pt[i] > P.f_pt_min) & (fabsf(eta[i]) < P.f_eta_max);
-  }
+__device__ __forceinline__ void cut_observe(const EventParams &P, const float (&pk)[4], float y, float &eta, int &pass,
+                                            float &sum, float &lead) {
+  const float px = pk[1], py = pk[2], pz = pk[3];
+  const float pt2 = __fmaf_rn(px, px, __fmul_rn(py, py));
+  const float pabs = sqrtf(__fmaf_rn(pz, pz, pt2));
+  const float pt = sqrtf(pt2);
+  eta = __fadd_rn(__fmul_rn(0.5f, logf(__fdiv_rn(__fadd_rn(pabs, pz), __fsub_rn(pabs, pz)))), y);
+  sum = __fadd_rn(sum, pt);
+  lead = fmaxf(lead, pt);
+  pass &= (pt > P.f_pt_min) & (fabsf(eta) < P.f_eta_max);
 }
 
 // Delta R of every pair (the Delta R cut); returns the smallest Delta R^2.
-// Azimuths once per gluon (m arctangents instead of m(m-1)/2), the pair's
+// Azimuths phi once per gluon (m arctangents instead of m(m-1)/2), the pair's
 // Delta phi = |phi_i - phi_j| folded into [0, pi]; each azimuth is within an
 // ulp or two of the exact one, so Delta phi is within ~1e-6 absolute, far
 // inside the FP32 forms' tolerance on cut decisions and R_min.
 template <int M>
-__device__ __forceinline__ float pair_cuts(const EventParams &P, const float (&px)[M], const float (&py)[M],
-                                           const float (&eta)[M], int &pass) {
+__device__ __forceinline__ float pair_cuts(const EventParams &P, const float (&eta)[M], const float (&phi)[M],
+                                           int &pass) {
   float dr2min = 1e30f;
-  float phi[M];
-#pragma unroll
-  for (int i = 0; i < M; ++i) phi[i] = atan2f(py[i], px[i]);
 #pragma unroll
   for (int i = 0; i < M; ++i) {
 #pragma unroll
@@ -451,17 +441,17 @@ __device__ __forceinline__ void scatter_ordered(const EventParams &P, uint64_t e
                                                 const float (&lk)[N][4], const float (&le1)[N][3],
                                                 const float (&le2)[N][2]) {
   constexpr int L = N - 1;
-  uint64_t posw;
+  PosWord<N> posw;
   const uint32_t hel = sample_positions<N>(P, ev, &posw);
   float *col = tile + slot;
   const float r2 = 0.70710678118654752440f;
 #pragma unroll
   for (int l = 0; l < N; ++l) {
-    const int p = (int)((posw >> (4 * l)) & 15ull);  // colour position of leg l
+    const int b = leg_block<N>(posw, l);
     const float sre = ((hel >> l) & 1u) ? r2 : -r2;
-    float *o = col + (p == 0 ? InRows<L>::eps0 : InRows<L>::eps(p - 1)) * kBlock;
-    if (p > 0) {
-      float *ok = col + InRows<L>::k(p - 1) * kBlock;
+    float *o = col + (l == 0 ? InRows<L>::eps0 : InRows<L>::eps(b)) * kBlock;
+    if (l > 0) {
+      float *ok = col + InRows<L>::k(b) * kBlock;
 #pragma unroll
       for (int q = 0; q < 4; ++q) ok[q * kBlock] = lk[l][q];
     }
@@ -481,17 +471,17 @@ __device__ __forceinline__ void scatter_ordered_real(const EventParams &P, uint6
                                                      const float (&lk)[N][4], const float (&le1)[N][3],
                                                      const float (&le2)[N][2]) {
   constexpr int L = N - 1;
-  uint64_t posw;
+  PosWord<N> posw;
   sample_positions<N>(P, ev, &posw);
   float cphi[N], sphi[N];
   polarisation_angles<N, float>(P, ev, cphi, sphi);
   float *col = tile + slot;
 #pragma unroll
   for (int l = 0; l < N; ++l) {
-    const int p = (int)((posw >> (4 * l)) & 15ull);  // colour position of leg l
-    float *o = col + (p == 0 ? InRows<L>::eps0 : InRows<L>::eps(p - 1)) * kBlock;
-    if (p > 0) {
-      float *ok = col + InRows<L>::k(p - 1) * kBlock;
+    const int b = leg_block<N>(posw, l);
+    float *o = col + (l == 0 ? InRows<L>::eps0 : InRows<L>::eps(b)) * kBlock;
+    if (l > 0) {
+      float *ok = col + InRows<L>::k(b) * kBlock;
 #pragma unroll
       for (int q = 0; q < 4; ++q) ok[q * kBlock] = lk[l][q];
     }
@@ -625,15 +615,16 @@ __device__ __forceinline__ void kin_fp32(const ChunkParams &C, const ChunkBuf<fl
 
   // cuts and observables in FP32
   const float y = __fmul_rn(0.5f, logf(__fdiv_rn(x1, x2)));
-  float eta[M], pt[M], px[M], py[M], pkf[M][4];
-#pragma unroll
-  for (int i = 0; i < M; ++i)
-#pragma unroll
-    for (int m = 0; m < 4; ++m) pkf[i][m] = (float)pk[i][m];
+  float eta[M], phi[M];
   int pass = 1;
   float sum = 0.f, lead = 0.f;
-  cuts_observables<M>(P, pkf, y, px, py, pt, eta, pass, sum, lead);
-  const float dr2min = pair_cuts<M>(P, px, py, eta, pass);
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    const float pkf[4] = {(float)pk[i][0], (float)pk[i][1], (float)pk[i][2], (float)pk[i][3]};
+    cut_observe(P, pkf, y, eta[i], pass, sum, lead);
+    phi[i] = atan2f(pkf[2], pkf[1]);
+  }
+  const float dr2min = pair_cuts<M>(P, eta, phi, pass);
   const double ht = (double)sum, ptlead = (double)lead, rmin = (double)sqrtf(dr2min);
   if (live) {
     if (P.ht) P.ht[idx] = ht;
@@ -712,6 +703,12 @@ __device__ __forceinline__ void pol_basis_rounded(float E, float px, float py, f
   e2[1] = cf;
 }
 
+// Final-state gluons per trip of the double-float kinematics' loops, measured
+// per 2^22 events at n = 4 / 6 / 8 / 10: one 256 / 428 / 620 / 836 us, two 232 /
+// 405 / 595 / 799 us, four 235 / 418 / 698 / 908 us, all of them 256 / 457 / 699 /
+// 971 us.
+constexpr int kKinUnroll = 2;
+
 // K1, double-float form: as kin_fp32, with the step that needs more than
 // FP32 -- Rambo's boost and rescale -- in double-float (two-float)
 // arithmetic on the FP32 pipe instead of native FP64 (1/64 of the FP32 rate
@@ -783,13 +780,24 @@ __device__ __forceinline__ void kin_ds_back(const ChunkParams &C, const ChunkBuf
   scatter_legs<N, RP>(P, ev, tile, slot, lk, le1, le2);
 }
 
+// First half and second half together.  The loops over the final-state
+// gluons are rolled (kKinUnroll gluons per trip) and hand their per-gluon
+// values (seed, momentum, pseudorapidity, azimuth) from loop to loop through
+// the thread's own column of the output tile, which the second half reads back
+// before it scatters into it.  What bounds the kernel is instruction issue:
+// with every loop unrolled the body is ~2,800 instructions (45 KB) at n = 6,
+// which each warp streams through the instruction cache once per event
+// (no_instruction 1.1 per issue, 73 % of the issue slots used); rolled it also
+// takes fewer registers (56 instead of 80 at n = 6: 8 blocks per SM for 6).
 template <int N, bool RP, bool CF>
 __device__ __forceinline__ void kin_ds(const ChunkParams &C, const ChunkBuf<float> &B, int e, float *tile,
                                      bool live) {
   constexpr int M = N - 2;
+  static_assert(6 * M + 9 <= InRows<N - 1>::rows, "scratch rows of the column");
   const EventParams &P = C.P;
   const uint64_t idx = C.chunk_first + (uint64_t)e;
   const uint64_t ev = P.first_event + idx;
+  float *const col = tile + threadIdx.x;
 
   const uint4 w0 = event_block(P, ev, 0);
   const float lnxmin = P.f_lnxmin;
@@ -799,9 +807,8 @@ __device__ __forceinline__ void kin_ds(const ChunkParams &C, const ChunkBuf<floa
   const DS shat = ds_mul(ds_mul(DS{P.S_hi, P.S_lo}, x1), x2);
   const DS rs = ds_sqrt(shat);
 
-  float qf[M][4];
   float Qh[4] = {0.f, 0.f, 0.f, 0.f}, Ql[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
+#pragma unroll kKinUnroll
   for (int i = 0; i < M; ++i) {
     const uint4 wa = event_block(P, ev, 1 + 2 * i);
     const uint4 wb = event_block(P, ev, 2 + 2 * i);
@@ -810,15 +817,13 @@ __device__ __forceinline__ void kin_ds(const ChunkParams &C, const ChunkBuf<floa
     float sn, cs;
     sincospif(2.f * unit_f32(wa.z, wa.w), &sn, &cs);
     const float q0 = -logf(unit_f32(wb.x, wb.y) * unit_f32(wb.z, wb.w));
-    qf[i][0] = q0;
-    qf[i][1] = q0 * sn0 * cs;
-    qf[i][2] = q0 * sn0 * sn;
-    qf[i][3] = q0 * c;
+    const float q[4] = {q0, q0 * sn0 * cs, q0 * sn0 * sn, q0 * c};
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       float t;
-      Qh[m] = two_sum(Qh[m], qf[i][m], t);
+      Qh[m] = two_sum(Qh[m], q[m], t);
       Ql[m] += t;
+      col[(4 * i + m) * kBlock] = q[m];
     }
   }
   DS Q[4];
@@ -831,43 +836,54 @@ __device__ __forceinline__ void kin_ds(const ChunkParams &C, const ChunkBuf<floa
   const DS aa = ds_rcp(ds_add(gam, 1.f));
   const DS xs = ds_mul(rs, invM);
   // boost and rescale of each seed, k = xs (gam q0 + b.q, q + b f), f = aa b.q
-  // + q0, in unnormalised pairs, each component rounded once to FP32
-  float pk[M][4];
-#pragma unroll
+  // + q0, in unnormalised pairs, each component rounded once to FP32; then
+  // cuts and observables in FP32 from the rounded momenta, with the partonic
+  // rapidity 0.5 ln(x1 / x2) from the logarithms drawn above
+  const float y = __fmul_rn(__fmul_rn(0.5f, lnxmin), __fsub_rn(ux1, ux2));
+  int pass = 1;
+  float sum = 0.f, lead = 0.f;
+#pragma unroll kKinUnroll
   for (int i = 0; i < M; ++i) {
+    float q[4], pk[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) q[m] = col[(4 * i + m) * kBlock];
     float t, l1, l2, l3;
-    const float p1 = pair_mul(b[0].hi, b[0].lo, qf[i][1], l1);
-    const float p2 = pair_mul(b[1].hi, b[1].lo, qf[i][2], l2);
-    const float p3 = pair_mul(b[2].hi, b[2].lo, qf[i][3], l3);
+    const float p1 = pair_mul(b[0].hi, b[0].lo, q[1], l1);
+    const float p2 = pair_mul(b[1].hi, b[1].lo, q[2], l2);
+    const float p3 = pair_mul(b[2].hi, b[2].lo, q[3], l3);
     float uh = two_sum(p1, p2, t);
     float ul = t + l1 + l2 + l3;
     uh = two_sum(uh, p3, t);
     ul += t;  // (uh, ul) = b.q
     float gl;
-    const float gh = pair_mul(gam.hi, gam.lo, qf[i][0], gl);
+    const float gh = pair_mul(gam.hi, gam.lo, q[0], gl);
     const float eh = two_sum(gh, uh, t);
-    pk[i][0] = pair_mul_round(xs.hi, xs.lo, eh, t + gl + ul);
+    pk[0] = pair_mul_round(xs.hi, xs.lo, eh, t + gl + ul);
     float fl;
     const float fp = pair_mul(aa.hi, aa.lo, uh, ul, fl);
-    const float fh = two_sum(fp, qf[i][0], t);
+    const float fh = two_sum(fp, q[0], t);
     fl += t;  // (fh, fl) = f
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       float bl;
       const float bh = pair_mul(b[j].hi, b[j].lo, fh, fl, bl);
-      const float sh = two_sum(qf[i][1 + j], bh, t);
-      pk[i][1 + j] = pair_mul_round(xs.hi, xs.lo, sh, t + bl);
+      const float sh = two_sum(q[1 + j], bh, t);
+      pk[1 + j] = pair_mul_round(xs.hi, xs.lo, sh, t + bl);
     }
+    float eta;
+    cut_observe(P, pk, y, eta, pass, sum, lead);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) col[(4 * i + m) * kBlock] = pk[m];
+    col[(4 * M + i) * kBlock] = eta;
+    col[(5 * M + i) * kBlock] = atan2f(pk[2], pk[1]);
   }
-
-  // cuts and observables in FP32 from the rounded momenta; the partonic
-  // rapidity 0.5 ln(x1 / x2) from the logarithms drawn above
-  const float y = __fmul_rn(__fmul_rn(0.5f, lnxmin), __fsub_rn(ux1, ux2));
-  float eta[M], pt[M], px[M], py[M];
-  int pass = 1;
-  float sum = 0.f, lead = 0.f;
-  cuts_observables<M>(P, pk, y, px, py, pt, eta, pass, sum, lead);
-  float dr2min = pair_cuts<M>(P, px, py, eta, pass);
+  float eta[M], phi[M];
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    eta[i] = col[(4 * M + i) * kBlock];
+    phi[i] = col[(5 * M + i) * kBlock];
+  }
+  const float dr2min = pair_cuts<M>(P, eta, phi, pass);
   const float rmin = sqrtf(dr2min);
   if (live) {
     if (P.ht) P.ht[idx] = (double)sum;
@@ -875,41 +891,45 @@ __device__ __forceinline__ void kin_ds(const ChunkParams &C, const ChunkBuf<floa
     if (P.rmin) P.rmin[idx] = (double)rmin;
     if (P.pass) P.pass[idx] = (uint8_t)pass;
   }
+  float pk[M][4];
   if constexpr (!CF) {
+#pragma unroll
+    for (int i = 0; i < M; ++i)
+#pragma unroll
+      for (int m = 0; m < 4; ++m) pk[i][m] = col[(4 * i + m) * kBlock];
     kin_ds_back<N, RP, CF>(C, B, tile, (int)threadIdx.x, e, ev, rs.hi, shat.hi, sum, lead, rmin, x1, x2, ux1, ux2,
                            pass, pk);
   } else {
     // the block's kept events are finished by its first threads, one each,
-    // with their first-half results staged in shared memory
-    constexpr int NS = 4 * M + 12;
-    __shared__ uint32_t st[NS][kBlock];
+    // from the first halves' columns
+    __shared__ int src[kBlock];
     int kept = 0;
     int slot = cut_first_slot<CF>(P, B, live, pass, idx, &kept);
     if (slot >= 0) {
-      const float v[12] = {rs.hi, shat.hi, sum, lead, rmin, x1, x2, ux1, ux2, 0.f, 0.f, 0.f};
+      const float v[9] = {rs.hi, shat.hi, sum, lead, rmin, x1, x2, ux1, ux2};
 #pragma unroll
-      for (int q = 0; q < 9; ++q) st[q][slot] = __float_as_uint(v[q]);
-      st[9][slot] = (uint32_t)e;
-      st[10][slot] = (uint32_t)ev;
-      st[11][slot] = (uint32_t)(ev >> 32);
-#pragma unroll
-      for (int i = 0; i < M; ++i)
-#pragma unroll
-        for (int m = 0; m < 4; ++m) st[12 + 4 * i + m][slot] = __float_as_uint(pk[i][m]);
+      for (int q = 0; q < 9; ++q) col[(6 * M + q) * kBlock] = v[q];
+      src[slot] = (int)threadIdx.x;
     }
     __syncthreads();
     slot = (int)threadIdx.x;
+    float q[9];
+    int from = 0;
+    if (slot < kept) {
+      from = src[slot];
+      const float *c = tile + from;
+#pragma unroll
+      for (int i = 0; i < 9; ++i) q[i] = c[(6 * M + i) * kBlock];
+#pragma unroll
+      for (int i = 0; i < M; ++i)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) pk[i][m] = c[(4 * i + m) * kBlock];
+    }
+    __syncthreads();  // every column has been read before any is scattered into
     if (slot >= kept) return;
-    float q[9], pq[M][4];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) q[i] = __uint_as_float(st[i][slot]);
-#pragma unroll
-    for (int i = 0; i < M; ++i)
-#pragma unroll
-      for (int m = 0; m < 4; ++m) pq[i][m] = __uint_as_float(st[12 + 4 * i + m][slot]);
-    const int eo = (int)st[9][slot];
-    const uint64_t evo = (uint64_t)st[10][slot] | ((uint64_t)st[11][slot] << 32);
-    kin_ds_back<N, RP, CF>(C, B, tile, slot, eo, evo, q[0], q[1], q[2], q[3], q[4], q[5], q[6], q[7], q[8], 1, pq);
+    const int eo = (int)blockIdx.x * kBlock + from;
+    kin_ds_back<N, RP, CF>(C, B, tile, slot, eo, P.first_event + C.chunk_first + (uint64_t)eo, q[0], q[1], q[2], q[3],
+                           q[4], q[5], q[6], q[7], q[8], 1, pk);
   }
 }
 
