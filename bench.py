@@ -294,10 +294,12 @@ def bench_config(torch, tess, ctx, name, flush, steps, peaks, sm_mhz, autotune=T
             tess.tess_autotune(ctx, proc, min(ne, 1 << 25), None, run.workspace, outputs=run.outputs)
         ms = statistics.mean(time_steps(torch, run, 1, 0, steps, 2, flush))
         amp_ms, amp_launches, plan, _ = amp_kernel_time(torch, tess, ctx, proc, run, 1, 0, flush, steps)
-        # the exact sum evaluates (n-1)! orderings x 2^(n-1) helicity labellings per event (flipping every
-        # label leaves |m| unchanged, so leg 0 keeps label 0 and the sum is doubled)
-        evals = ne * (math.factorial(n - 1) * 2 ** (n - 1) if wl["hel"] == "sum" else 1)
-        fl = tess.flops_per_event(n, plan["variant"], precision=proc.precision)  # as the timed variant evaluates it
+        # FLOPs as the timed variant evaluates them (the exact sum: every amplitude that is neither equal to
+        # another nor zero)
+        exact = wl["hel"] == "sum"
+        evals = ne * (tess.exact_sum_amplitudes(n) if exact else 1)
+        fl = (tess.exact_sum_flops(n) / tess.exact_sum_amplitudes(n) if exact
+              else tess.flops_per_event(n, plan["variant"], precision=proc.precision))
         achieved = fl * evals / (amp_ms * 1e-3) / 1e12
         pk = peak_at(peaks, "fp64" if form == "fp64" else "fp32", sm_mhz)
         sg = run.result()
@@ -591,8 +593,9 @@ def run_tess(args):
             amp_ms, amp_launches = stages["fused"]
         amp_ms_step = amp_ms / args.steps
         evaluated = n_pass_local if cf else N  # amplitudes computed per step (cut-first: passing events)
-        if wl["hel"] == "sum":  # every colour ordering and helicity labelling of each event (leg 0's label fixed)
-            evaluated = N * math.factorial(n - 1) * 2 ** (n - 1)
+        if wl["hel"] == "sum":  # every amplitude of an event that is neither equal to another nor zero
+            evaluated = N * tess.exact_sum_amplitudes(n)
+            flops_per_event = tess.exact_sum_flops(n) / tess.exact_sum_amplitudes(n)
         achieved = flops_per_event * evaluated / (amp_ms_step * 1e-3) / 1e12
         tot = sum(v[0] for v in stages.values()) or 1.0
         traffic = read_traffic(args.workload + ("_rp" if rp else "") + ("_cf" if cf else ""), plan["variant"],

@@ -576,9 +576,10 @@ def bg_flops_real_leaf(n):
 
 def flops_per_event(n, variant, random_pol=False, precision=None):
     """FLOPs of one amplitude as the given amplitude variant evaluates it
-    (variant -1: the exact-sum mode's fused kernel, whose recursion is the
-    register form for FP32 up to n = 7 and FP64 up to n = 5, else the loop
-    form; pass the process's precision)."""
+    (variant -1: the one-kernel-per-event form of tess_generate_noalloc's sampled
+    events, whose recursion is the register form for FP32 up to n = 7 and FP64 up
+    to n = 5, else the loop form; pass the process's precision.  The exact sum:
+    exact_sum_flops)."""
     if variant == -1 and not random_pol:
         reg = n <= 7 if precision in (TESS_FP32_CURRENTS, TESS_FP32_DS) else n <= 5
         return bg_flops_leaf(n) if reg else bg_flops(n)
@@ -592,6 +593,58 @@ def flops_per_event(n, variant, random_pol=False, precision=None):
     if variant == 15:  # TESS_K2_WAVE2U
         return bg_flops_wave_unrolled(n)
     return bg_flops_wave(n) if variant in WAVE_FORMS else bg_flops(n)
+
+
+def _lc_order_flops(L):
+    """Momenta's part of one ordering in light-cone gauge (tess_lc.cuh lc_order):
+    the sums of K+ before and after each leg, the second incoming leg's K+, and
+    per set K+, K-, K_perp, the incoming and outgoing form of K^2, one reciprocal
+    and b."""
+    sets = L * (L - 1) // 2 - 1
+    return 2 * L + L + sets * (5 + 6 + 10 + 1 + 6)
+
+
+def _lc_amplitude_flops(L):
+    """One labelling of an ordering in light-cone gauge (tess_lc.cuh
+    lc_amplitude)."""
+    def dot(la, lb):
+        return 2 if la and lb else (4 if la or lb else 16)
+
+    total = 0
+    for ln in range(2, L):
+        for a in range(0, L - ln + 1):
+            b = a + ln - 1
+            for i in range(a, b):
+                ll, lr = i == a, i + 1 == b
+                total += 2 + dot(ll, lr)                          # db, D
+                total += (4 if ll else 13) + (4 if lr else 13)    # c_r, c_l
+                total += (6 if lr else 16) + (6 if ll else 16)    # c_r J_r, c_l J_l
+                total += 5 + 8 + 2 + 1 + 4                        # D db term, S, w
+                for j in range(i + 1, b):                         # triples ([a..i], [i+1..j], [j+1..b])
+                    total += dot(i == a, j + 1 == b) + (6 if j == i + 1 else 16)
+            total += 12 + 8                                       # propagator; w, A, B, omega
+    e = L - 1
+    for i in range(0, e):
+        total += (8 + dot(i + 1 == e, True) if i > 0 else 0) + (8 + dot(i == 0, True) if i + 1 < e else 0)
+        total += 3 + 8 + dot(i == 0, i + 1 == e)
+        for j in range(i + 1, e):
+            total += 8 + dot(i == 0, j + 1 == e) + dot(j == i + 1, True)
+    return total + 4
+
+
+def exact_sum_flops(n):
+    """Real floating-point operations of one event's exact sum over helicities
+    and colour orderings (n = 4, 5) as the kernel evaluates it: half of the
+    (n-1)! orderings (the reversed ones are equal), of each the 2^(n-1) labellings
+    with leg 0's label fixed that do not vanish at tree level."""
+    L = n - 1
+    orderings = math.factorial(n - 1) // 2
+    return orderings * _lc_order_flops(L) + exact_sum_amplitudes(n) * (_lc_amplitude_flops(L) + 4)
+
+
+def exact_sum_amplitudes(n):
+    """Amplitudes that the exact sum evaluates per event: 9 at n = 4, 120 at n = 5."""
+    return math.factorial(n - 1) // 2 * sum(math.comb(n - 1, k) for k in range(2, n - 1))
 
 
 def bg_flops_real(n):

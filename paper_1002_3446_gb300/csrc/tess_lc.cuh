@@ -1,0 +1,260 @@
+// Berends-Giele recursion (Sec. 3) in light-cone gauge, for the exact sum over
+// helicities and colour orderings.
+//
+// The amplitude does not depend on the gauge of the polarisation vectors and
+// propagators.  With the reference vector q along the incoming gluon of leg 0
+// (which every ordering contracts last), q.J = 0 for every current, so that a
+// current has two transverse components J = (J_x, J_y) instead of four, and
+// J.J' = -(J_x J'_x + J_y J'_y).  Notation for a set X of legs: K+ = K^0 - K^3
+// (its component along q), b = K_perp / K+, D = J_l.J_r over the transverse
+// components of a split's parts, and the scalars
+//   S_X = sum_splits D,  w_X = sum_splits D (K_l+ - K_r+) / K_X+,
+//   A = S + w,  B = S - w,  omega = w / K+
+// (S is the reorganised four-gluon vertex of tess_bg.cuh, w the instantaneous
+// part of the light-cone propagator).  Then
+//   K_X^2 J_X = sum_splits [ c_r J_r + c_l J_l - (2 K_l+ K_r+ / K_X+) D db ]
+//               - 2 sum_triples (J_A.J_C) J_B,
+//   c_r = 2 K_r+ (J_l.db + omega_l) + A_l,  c_l = 2 K_l+ (J_r.db - omega_r) + B_r,
+//   db = b_l - b_r,
+// and in the last current, whose K+ vanishes with db,
+//   t = sum_splits [ B_l e0.J_r + A_r e0.J_l - 2 D e0.K_l ] - 2 sum_triples (J_A.J_C) e0.J_B.
+// A gluon's polarisation vector is (1, i s) / sqrt2 up to a phase, s = -1 for
+// helicity label 0 and +1 for label 1 (opposite for leg 0), whatever its
+// momentum, so the momenta's part of an ordering is shared by its helicities.
+//
+// K+ is a sum of positive numbers for sets of outgoing legs, and minus the
+// sum over the other outgoing legs for a set with the second incoming leg
+// (K+ of all legs but leg 0 is zero), so nothing cancels in it, and the same
+// holds for K^2: K^2 / K+ of a set grows by |db|^2 K_l+ K_r+ / K_X+ with each
+// outgoing leg, and is -(K+_rest K-_out + K_perp^2) / K+ with the incoming one.
+#pragma once
+#include "tess_math.cuh"
+
+namespace tess {
+
+// One leg of 1..N-1: transverse momentum, K+ and K- (zero for the second
+// incoming leg, see LCOrder) and b.
+template <typename R>
+struct LCLeg {
+  R x, y, p, m, bx, by;
+};
+
+// Light-cone components of an outgoing massless momentum: the smaller of K+,
+// K- from pT^2 over the larger.
+template <typename R>
+__device__ __forceinline__ LCLeg<R> lc_leg(double e, double px, double py, double pz) {
+  const double pt2 = px * px + py * py, big = e + fabs(pz), small = pt2 / big;
+  const double p = pz > 0.0 ? small : big, ip = pz > 0.0 ? big / pt2 : 1.0 / big;
+  return {R(px), R(py), R(p), R(pz > 0.0 ? big : small), R(px * ip), R(py * ip)};
+}
+
+// What the sets [a..b] (1 < length < L) and legs of one ordering need of the
+// momenta: K+, b, 1 / K+ and 1 / K^2; and K_perp of the sets [0..i].
+template <typename R, int L>
+struct LCOrder {
+  R p[L][L], bx[L][L], by[L][L], ip[L][L], ik2[L][L], kx[L], ky[L];
+};
+
+// g: the legs in colour order; two: position of the second incoming leg.
+template <typename R, int L>
+__device__ __forceinline__ void lc_order(const LCLeg<R> (&g)[L], int two, LCOrder<R, L> &o) {
+  R pre[L + 1], suf[L + 1];  // K+ of the outgoing legs before a / from a on
+  pre[0] = R(0);
+  suf[L] = R(0);
+#pragma unroll
+  for (int a = 0; a < L; ++a) pre[a + 1] = pre[a] + g[a].p;
+#pragma unroll
+  for (int a = L - 1; a >= 0; --a) suf[a] = suf[a + 1] + g[a].p;
+  o.kx[0] = g[0].x;
+  o.ky[0] = g[0].y;
+#pragma unroll
+  for (int a = 0; a < L; ++a) {
+    o.p[a][a] = a == two ? -(pre[a] + suf[a + 1]) : g[a].p;
+    o.bx[a][a] = g[a].bx;
+    o.by[a][a] = g[a].by;
+  }
+#pragma unroll
+  for (int a = 0; a < L; ++a) {
+    R wp = g[a].p, wm = g[a].m, x = g[a].x, y = g[a].y, mass = R(0);
+#pragma unroll
+    for (int b = a + 1; b < L; ++b) {
+      if (a == 0 && b == L - 1) break;
+      wp += g[b].p;
+      wm += g[b].m;
+      x += g[b].x;
+      y += g[b].y;
+      const bool in = a <= two && two <= b;
+      const R rest = pre[a] + suf[b + 1];
+      const R p = in ? -rest : wp;
+      // 1 / K+ and 1 / K^2 from one reciprocal; outgoing legs: K^2 / K+ =
+      // mass' = mass + |db|^2 p_l p_r / p, so K^2 = p mass + |db|^2 p_l p_r
+      const R dx = o.bx[a][b - 1] - o.bx[b][b], dy = o.by[a][b - 1] - o.by[b][b];
+      const R k2 = in ? -(rest * wm + (x * x + y * y)) : p * mass + (dx * dx + dy * dy) * (o.p[a][b - 1] * g[b].p);
+      const R r = R(1) / (p * k2);
+      o.ip[a][b] = r * k2;
+      o.ik2[a][b] = r * p;
+      mass = k2 * o.ip[a][b];
+      o.p[a][b] = p;
+      o.bx[a][b] = x * o.ip[a][b];
+      o.by[a][b] = y * o.ip[a][b];
+      if (a == 0) {
+        o.kx[b] = x;
+        o.ky[b] = y;
+      }
+    }
+  }
+}
+
+// A current: its transverse components.
+template <typename R>
+struct LCCur {
+  Cx<R> x, y;
+};
+
+// J.J' over the transverse components; a leaf is (1, i s).
+template <typename R>
+__device__ __forceinline__ Cx<R> lc_dot(const LCCur<R> &a, const LCCur<R> &b) {
+  R re = a.x.re * b.x.re, im = a.x.re * b.x.im;
+  re = fma(-a.x.im, b.x.im, re);
+  im = fma(a.x.im, b.x.re, im);
+  re = fma(a.y.re, b.y.re, re);
+  im = fma(a.y.re, b.y.im, im);
+  re = fma(-a.y.im, b.y.im, re);
+  im = fma(a.y.im, b.y.re, im);
+  return {re, im};
+}
+
+template <typename R>
+__device__ __forceinline__ Cx<R> lc_leaf_dot(R s, const LCCur<R> &b) {
+  return {fma(-s, b.y.im, b.x.re), fma(s, b.y.re, b.x.im)};
+}
+
+// acc += c v
+template <typename R>
+__device__ __forceinline__ void lc_axpy(LCCur<R> &acc, const Cx<R> &c, const LCCur<R> &v) {
+  acc.x.re = fma(c.re, v.x.re, acc.x.re);
+  acc.x.im = fma(c.re, v.x.im, acc.x.im);
+  acc.y.re = fma(c.re, v.y.re, acc.y.re);
+  acc.y.im = fma(c.re, v.y.im, acc.y.im);
+  acc.x.re = fma(-c.im, v.x.im, acc.x.re);
+  acc.x.im = fma(c.im, v.x.re, acc.x.im);
+  acc.y.re = fma(-c.im, v.y.im, acc.y.re);
+  acc.y.im = fma(c.im, v.y.re, acc.y.im);
+}
+
+// acc += c (1, i s)
+template <typename R>
+__device__ __forceinline__ void lc_axpy_leaf(LCCur<R> &acc, const Cx<R> &c, R s) {
+  acc.x.re += c.re;
+  acc.x.im += c.im;
+  acc.y.re = fma(-s, c.im, acc.y.re);
+  acc.y.im = fma(s, c.re, acc.y.im);
+}
+
+// t of the last current for the helicity signs s[a] of the colour positions
+// and s0 of leg 0: |m|^2 = |t|^2 / 2^(L+1) (paper normalisation; the factors
+// 1 / sqrt2 of the polarisation vectors).
+template <typename R, int L>
+__device__ __forceinline__ Cx<R> lc_amplitude(const LCOrder<R, L> &o, const R (&s)[L], R s0) {
+  LCCur<R> J[L][L];
+  Cx<R> A[L][L], B[L][L], om[L][L];
+  const Cx<R> zero = {R(0), R(0)};
+  auto dot = [&](int a, int b, int c, int d) {  // J[a..b].J[c..d]
+    if (a == b && c == d) return Cx<R>{fma(-s[a], s[c], R(1)), R(0)};
+    if (a == b) return lc_leaf_dot(s[a], J[c][d]);
+    if (c == d) return lc_leaf_dot(s[c], J[a][b]);
+    return lc_dot(J[a][b], J[c][d]);
+  };
+#pragma unroll
+  for (int len = 2; len < L; ++len) {
+#pragma unroll
+    for (int a = 0; a + len - 1 < L; ++a) {
+      const int b = a + len - 1;
+      LCCur<R> acc = {zero, zero}, tri = {zero, zero};
+      Cx<R> S = zero, w = zero;
+#pragma unroll
+      for (int i = a; i < b; ++i) {
+        const bool ll = i == a, lr = i + 1 == b;
+        const R pl = o.p[a][i], pr = o.p[i + 1][b];
+        const R dx = o.bx[a][i] - o.bx[i + 1][b], dy = o.by[a][i] - o.by[i + 1][b];
+        const Cx<R> D = dot(a, i, i + 1, b);
+        Cx<R> cr, cl;
+        if (ll) {
+          cr = {(R(2) * pr) * dx, (R(2) * pr) * (s[a] * dy)};
+        } else {
+          const LCCur<R> &l = J[a][i];
+          cr = {fma(R(2) * pr, fma(l.x.re, dx, fma(l.y.re, dy, om[a][i].re)), A[a][i].re),
+                fma(R(2) * pr, fma(l.x.im, dx, fma(l.y.im, dy, om[a][i].im)), A[a][i].im)};
+        }
+        if (lr) {
+          cl = {(R(2) * pl) * dx, (R(2) * pl) * (s[b] * dy)};
+        } else {
+          const LCCur<R> &r = J[i + 1][b];
+          cl = {fma(R(2) * pl, fma(r.x.re, dx, fma(r.y.re, dy, -om[i + 1][b].re)), B[i + 1][b].re),
+                fma(R(2) * pl, fma(r.x.im, dx, fma(r.y.im, dy, -om[i + 1][b].im)), B[i + 1][b].im)};
+        }
+        if (lr)
+          lc_axpy_leaf(acc, cr, s[b]);
+        else
+          lc_axpy(acc, cr, J[i + 1][b]);
+        if (ll)
+          lc_axpy_leaf(acc, cl, s[a]);
+        else
+          lc_axpy(acc, cl, J[a][i]);
+        const R gp = R(-2) * (pl * pr) * o.ip[a][b], gx = gp * dx, gy = gp * dy;
+        acc.x.re = fma(gx, D.re, acc.x.re);
+        acc.x.im = fma(gx, D.im, acc.x.im);
+        acc.y.re = fma(gy, D.re, acc.y.re);
+        acc.y.im = fma(gy, D.im, acc.y.im);
+        S.re += D.re;
+        S.im += D.im;
+        const R dp = pl - pr;
+        w.re = fma(dp, D.re, w.re);
+        w.im = fma(dp, D.im, w.im);
+      }
+#pragma unroll
+      for (int i = a; i + 1 < b; ++i) {
+#pragma unroll
+        for (int j = i + 1; j < b; ++j) {
+          const Cx<R> x = dot(a, i, j + 1, b);
+          if (j == i + 1)
+            lc_axpy_leaf(tri, x, s[j]);
+          else
+            lc_axpy(tri, x, J[i + 1][j]);
+        }
+      }
+      const R ik = o.ik2[a][b], ip = o.ip[a][b];
+      J[a][b].x = {fma(R(-2), tri.x.re, acc.x.re) * ik, fma(R(-2), tri.x.im, acc.x.im) * ik};
+      J[a][b].y = {fma(R(-2), tri.y.re, acc.y.re) * ik, fma(R(-2), tri.y.im, acc.y.im) * ik};
+      w = {w.re * ip, w.im * ip};
+      A[a][b] = {S.re + w.re, S.im + w.im};
+      B[a][b] = {S.re - w.re, S.im - w.im};
+      om[a][b] = {w.re * ip, w.im * ip};
+    }
+  }
+  // e0.J of the sets that the last current adds up
+  auto e0 = [&](int a, int b) {
+    if (a == b) return Cx<R>{fma(-s0, s[a], R(1)), R(0)};
+    return lc_leaf_dot(s0, J[a][b]);
+  };
+  constexpr int e = L - 1;
+  Cx<R> t = zero, tri = zero;
+  auto madd = [](Cx<R> &z, const Cx<R> &u, const Cx<R> &v) {
+    z.re = fma(u.re, v.re, fma(-u.im, v.im, z.re));
+    z.im = fma(u.re, v.im, fma(u.im, v.re, z.im));
+  };
+#pragma unroll
+  for (int i = 0; i < e; ++i) {
+    if (i > 0) madd(t, B[0][i], e0(i + 1, e));
+    if (i + 1 < e) madd(t, A[i + 1][e], e0(0, i));
+    const R kx = R(-2) * o.kx[i], ky = s0 * (R(-2) * o.ky[i]);
+    madd(t, dot(0, i, i + 1, e), Cx<R>{kx, ky});
+  }
+#pragma unroll
+  for (int i = 0; i + 1 < e; ++i)
+#pragma unroll
+    for (int j = i + 1; j < e; ++j) madd(tri, dot(0, i, j + 1, e), e0(i + 1, j));
+  return {fma(R(-2), tri.re, t.re), fma(R(-2), tri.im, t.im)};
+}
+
+}  // namespace tess
