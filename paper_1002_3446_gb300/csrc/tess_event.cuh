@@ -80,100 +80,6 @@ __device__ __forceinline__ void polarisations(T px, T py, T pz, CV4<R> &ep, CV4<
   }
 }
 
-// Phase space and phase-space weight stages.  Fills the all-outgoing momenta
-// kk[N][4] (k1 = -p1, k2 = -p2), the observables and the pass flag.
-template <int N>
-struct Kinematics {
-  static constexpr int M = N - 2;
-  double kk[N][4];
-  double x1, x2, shat, ht, ptlead, rmin;
-  int pass;
-};
-
-template <int N>
-__device__ __forceinline__ void kinematics(const EventParams &P, uint64_t ev, Kinematics<N> &K) {
-  constexpr int M = N - 2;
-  const double2 ux = uniform_pair(P.seed, ev, 0);
-  K.x1 = exp(ux.x * P.lnxmin);
-  K.x2 = exp(ux.y * P.lnxmin);
-  K.shat = K.x1 * K.x2 * P.S;
-  const double rs = sqrt(K.shat);
-  // Rambo (Kleiss-Stirling-Ellis): isotropic massless seeds q with energy
-  // density q0 exp(-q0), then one boost + rescale to total (rs, 0, 0, 0).
-  double q[M][4];
-  double Q0 = 0.0, Q1 = 0.0, Q2 = 0.0, Q3 = 0.0;
-#pragma unroll
-  for (int i = 0; i < M; ++i) {
-    const double2 a = uniform_pair(P.seed, ev, 1 + 2 * i);
-    const double2 b = uniform_pair(P.seed, ev, 2 + 2 * i);
-    const double c = 2.0 * a.x - 1.0;
-    const double s = sqrt(1.0 - c * c);
-    double sn, cs;
-    sincospi(2.0 * a.y, &sn, &cs);
-    const double q0 = -log(b.x * b.y);
-    q[i][0] = q0;
-    q[i][1] = q0 * s * cs;
-    q[i][2] = q0 * s * sn;
-    q[i][3] = q0 * c;
-    Q0 += q[i][0];
-    Q1 += q[i][1];
-    Q2 += q[i][2];
-    Q3 += q[i][3];
-  }
-  const double Mq = sqrt(Q0 * Q0 - Q1 * Q1 - Q2 * Q2 - Q3 * Q3);
-  const double invM = 1.0 / Mq;
-  const double bx = -Q1 * invM, by = -Q2 * invM, bz = -Q3 * invM;
-  const double gam = Q0 * invM;
-  const double aa = 1.0 / (1.0 + gam);
-  const double xs = rs * invM;
-  const double h = 0.5 * rs;
-  K.kk[0][0] = -h; K.kk[0][1] = 0.0; K.kk[0][2] = 0.0; K.kk[0][3] = -h;
-  K.kk[1][0] = -h; K.kk[1][1] = 0.0; K.kk[1][2] = 0.0; K.kk[1][3] = h;
-#pragma unroll
-  for (int i = 0; i < M; ++i) {
-    const double bq = bx * q[i][1] + by * q[i][2] + bz * q[i][3];
-    K.kk[2 + i][0] = xs * (gam * q[i][0] + bq);
-    const double f = aa * bq + q[i][0];
-    K.kk[2 + i][1] = xs * (q[i][1] + bx * f);
-    K.kk[2 + i][2] = xs * (q[i][2] + by * f);
-    K.kk[2 + i][3] = xs * (q[i][3] + bz * f);
-  }
-  // jets: every final-state gluon; lab rapidity = eta + ln(x1/x2)/2
-  const double y = 0.5 * log(K.x1 / K.x2);
-  double eta[M], pt[M];
-  int pass = 1;
-  double sum = 0.0, lead = 0.0;
-#pragma unroll
-  for (int i = 0; i < M; ++i) {
-    const double px = K.kk[2 + i][1], py = K.kk[2 + i][2], pz = K.kk[2 + i][3];
-    const double pt2 = px * px + py * py;
-    const double pabs = sqrt(pt2 + pz * pz);
-    pt[i] = sqrt(pt2);
-    eta[i] = 0.5 * log((pabs + pz) / (pabs - pz)) + y;
-    sum += pt[i];
-    lead = fmax(lead, pt[i]);
-    pass &= (pt[i] > P.pt_min) & (fabs(eta[i]) < P.eta_max);
-  }
-  double dr2min = 1.0e300;
-#pragma unroll
-  for (int i = 0; i < M; ++i) {
-#pragma unroll
-    for (int j = i + 1; j < M; ++j) {
-      const double pxi = K.kk[2 + i][1], pyi = K.kk[2 + i][2];
-      const double pxj = K.kk[2 + j][1], pyj = K.kk[2 + j][2];
-      const double dphi = atan2(fabs(pxi * pyj - pyi * pxj), pxi * pxj + pyi * pyj);
-      const double de = eta[i] - eta[j];
-      const double dr2 = de * de + dphi * dphi;
-      dr2min = fmin(dr2min, dr2);
-      pass &= (dr2 > P.dr2_min);
-    }
-  }
-  K.ht = sum;
-  K.ptlead = lead;
-  K.rmin = sqrt(dr2min);
-  K.pass = pass;
-}
-
 // Colour ordering (Fisher-Yates on positions 2..n) and helicity labels of a
 // sampled event, from its draws.  Both are integer functions of the Philox
 // words: the helicity word is the top n bits of its uniform, and each swap
@@ -184,6 +90,222 @@ __device__ __forceinline__ uint4 event_block(const EventParams &P, uint64_t ev, 
   return philox4x32_10_rk(make_uint4((uint32_t)ev, (uint32_t)(ev >> 32), blk, 0u), P.rk);
 }
 
+// x 2^s by adding s to the exponent field: equal to ldexp(x, s) for a normal
+// nonzero x whose result is normal (the callers' factors are far inside the
+// double range), in two integer operations instead of FP64 work.
+__device__ __forceinline__ double scale_pow2(double x, int s) {
+  return __longlong_as_double(__double_as_longlong(x) + ((long long)s << 52));
+}
+
+// The same for an x that may be zero.
+__device__ __forceinline__ double scale_pow2_z(double x, int s) {
+  const long long b = __double_as_longlong(x);
+  return (b << 1) == 0 ? x : __longlong_as_double(b + ((long long)s << 52));
+}
+
+// e with x = f 2^e, f in [1/2, 1), of a positive normal x.
+__device__ __forceinline__ int exponent_of(double x) {
+  return (int)((uint64_t)__double_as_longlong(x) >> 52) - 1022;
+}
+
+// e^eta of a massless momentum as n / d, without cancellation.
+__device__ __forceinline__ void exp_eta(double pt, double pz, double &n, double &d) {
+  const double big = sqrt(pt * pt + pz * pz) + fabs(pz);
+  n = pz > 0.0 ? big : pt;
+  d = pz > 0.0 ? pt : big;
+}
+
+// FP64 kinematics.  The FP64 pipe (1/64 of the FP32 rate) bounds every kernel
+// that runs them, so what the results do not need in 64 bits is not computed
+// there: the pseudorapidity cut and the pair with the smallest Delta R are
+// found in FP32 with an error bound, and FP64 decides whatever lies within it.
+//
+// FP32 estimates, absolute errors: eta (|eta| < 30) within 4e-6 (logarithm of a
+// ratio good to 5 ulp, rounding of a value up to 30), phi within 1e-6, so a
+// pair's Delta R within 6e-6 including its own rounding; kEstimate covers two
+// such errors and the conversion of the cut.
+constexpr float kEstimate = 2e-5f;
+
+// Phase space and phase-space weight stages: the final-state momenta k (the
+// incoming legs are k_0 = (-h, 0, 0, -h), k_1 = (-h, 0, 0, h), h = rs / 2), their
+// pT^2 and pT, the observables, the pass flag, and the weight over the
+// matrix-element estimator E (0 if the event fails the cuts).
+template <int N>
+struct Kinematics {
+  static constexpr int M = N - 2;
+  double k[M][4], pt2[M], pt[M];
+  double rs, ht, ptlead, rmin, wf;
+  int pass;
+};
+
+template <int N>
+__device__ __forceinline__ void kinematics(const EventParams &P, uint64_t ev, Kinematics<N> &K) {
+  constexpr int M = N - 2;
+  auto pair = [&](uint32_t blk, double &u0, double &u1) {
+    const uint4 w = event_block(P, ev, blk);
+    u0 = unit_from_words(w.x, w.y);
+    u1 = unit_from_words(w.z, w.w);
+  };
+  double u1, u2;
+  pair(0, u1, u2);
+  const double x1 = exp(u1 * P.lnxmin), x2 = exp(u2 * P.lnxmin);
+  const double shat = x1 * x2 * P.S;
+  K.rs = sqrt(shat);
+  // Rambo (Kleiss-Stirling-Ellis): isotropic massless seeds q with energy
+  // density q0 exp(-q0), then one boost + rescale to total (rs, 0, 0, 0).
+  double q[M][4];
+  double Q0 = 0.0, Q1 = 0.0, Q2 = 0.0, Q3 = 0.0;
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    double a1, a2, b1, b2;
+    pair(1 + 2 * i, a1, a2);
+    pair(2 + 2 * i, b1, b2);
+    const double c = 2.0 * a1 - 1.0;
+    const double s = sqrt(1.0 - c * c);
+    double sn, cs;
+    sincospi(2.0 * a2, &sn, &cs);
+    const double q0 = -log(b1 * b2), qs = q0 * s;
+    q[i][0] = q0;
+    q[i][1] = qs * cs;
+    q[i][2] = qs * sn;
+    q[i][3] = q0 * c;
+    Q0 += q[i][0];
+    Q1 += q[i][1];
+    Q2 += q[i][2];
+    Q3 += q[i][3];
+  }
+  const double invM = 1.0 / sqrt(Q0 * Q0 - Q1 * Q1 - Q2 * Q2 - Q3 * Q3);
+  const double bx = -Q1 * invM, by = -Q2 * invM, bz = -Q3 * invM;
+  const double gam = Q0 * invM;
+  const double aa = 1.0 / (1.0 + gam);
+  const double xs = K.rs * invM;
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    const double bq = bx * q[i][1] + by * q[i][2] + bz * q[i][3];
+    K.k[i][0] = xs * (gam * q[i][0] + bq);
+    const double f = aa * bq + q[i][0];
+    K.k[i][1] = xs * (q[i][1] + bx * f);
+    K.k[i][2] = xs * (q[i][2] + by * f);
+    K.k[i][3] = xs * (q[i][3] + bz * f);
+  }
+  // jets: every final-state gluon; lab rapidity = eta + ln(x1/x2)/2
+  const double y = 0.5 * P.lnxmin * (u1 - u2);
+  const float yf = (float)y, etamax = (float)P.eta_max;
+  float eta[M], phi[M];
+  uint32_t unsure = 0;  // gluons whose pseudorapidity FP64 has to decide
+  int pass = 1;
+  K.ht = 0.0;
+  K.ptlead = 0.0;
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    const double px = K.k[i][1], py = K.k[i][2];
+    K.pt2[i] = px * px + py * py;
+    K.pt[i] = sqrt(K.pt2[i]);
+    K.ht += K.pt[i];
+    K.ptlead = fmax(K.ptlead, K.pt[i]);
+    pass &= K.pt[i] > P.pt_min;
+    const float fx = (float)px, fy = (float)py, fz = (float)K.k[i][3];
+    const float ft = sqrtf(fmaf(fx, fx, fy * fy));
+    eta[i] = copysignf(logf((sqrtf(fmaf(fz, fz, ft * ft)) + fabsf(fz)) / ft), fz);
+    phi[i] = atan2f(fy, fx);
+    const float d = fabsf(eta[i] + yf) - etamax;
+    if (fabsf(d) > kEstimate && fabsf(eta[i]) < 30.f)
+      pass &= d < 0.f;
+    else
+      unsure |= 1u << i;
+  }
+  // momentum of gluon i, picked without dynamic register indexing
+  auto pick = [&](int i, double &px, double &py, double &pz, double &pt) {
+    px = K.k[0][1];
+    py = K.k[0][2];
+    pz = K.k[0][3];
+    pt = K.pt[0];
+#pragma unroll
+    for (int l = 1; l < M; ++l) {
+      px = i == l ? K.k[l][1] : px;
+      py = i == l ? K.k[l][2] : py;
+      pz = i == l ? K.k[l][3] : pz;
+      pt = i == l ? K.pt[l] : pt;
+    }
+  };
+  double pxi, pyi, pzi, pti, ni, di;
+  while (unsure) {
+    pick(__ffs((int)unsure) - 1, pxi, pyi, pzi, pti);
+    unsure &= unsure - 1;
+    exp_eta(pti, pzi, ni, di);
+    pass &= fabs(log(ni / di) + y) < P.eta_max;
+  }
+  // pairs that can have the smallest Delta R
+  auto estimate = [&](int i, int j) {
+    float dphi = fabsf(phi[i] - phi[j]);
+    dphi = dphi > 3.14159265f ? 6.28318531f - dphi : dphi;
+    const float de = eta[i] - eta[j];
+    return fmaf(de, de, dphi * dphi);
+  };
+  float least = 1e30f;
+#pragma unroll
+  for (int i = 0; i < M; ++i)
+#pragma unroll
+    for (int j = i + 1; j < M; ++j) least = fminf(least, estimate(i, j));
+  const float lim = sqrtf(least) + kEstimate, lim2 = lim * lim;
+  uint64_t near = 0;  // bit M i + j, i < j (an estimate that is no number: FP64 decides)
+  uint64_t near_hi = 0;
+#pragma unroll
+  for (int i = 0; i < M; ++i)
+#pragma unroll
+    for (int j = i + 1; j < M; ++j) {
+      const int bit = M * i + j;
+      const bool in = !(estimate(i, j) > lim2);
+      if (bit < 64)
+        near |= (uint64_t)in << (bit & 63);
+      else
+        near_hi |= (uint64_t)in << (bit & 63);
+    }
+  double dr2min = 1.0e300;
+  while (near | near_hi) {
+    int bit;
+    if (near) {
+      bit = __ffsll((long long)near) - 1;
+      near &= near - 1;
+    } else {
+      bit = 63 + __ffsll((long long)near_hi);
+      near_hi &= near_hi - 1;
+    }
+    double pxj, pyj, pzj, ptj, nj, dj;
+    pick(bit / M, pxi, pyi, pzi, pti);
+    pick(bit % M, pxj, pyj, pzj, ptj);
+    exp_eta(pti, pzi, ni, di);
+    exp_eta(ptj, pzj, nj, dj);
+    const double dphi = atan2(fabs(pxi * pyj - pyi * pxj), pxi * pxj + pyi * pyj);
+    const double de = log((ni * dj) / (di * nj));
+    const double dr2 = de * de + dphi * dphi;
+    dr2min = fmin(dr2min, dr2);
+    pass &= dr2 > P.dr2_min;
+  }
+  K.rmin = sqrt(dr2min);
+  K.pass = pass;
+  K.wf = 0.0;
+  if (pass) {
+    const double mu = P.mu_r_factor * K.ht;
+    const double as = P.alphas_mz / (1.0 + P.alphas_mz * P.b0 * (log(mu * mu) - P.ln_mz2));
+    const double g2 = 4.0 * 3.14159265358979323846 * as;
+    // f(x1) f(x2) with f(x) = 1.7 x^-0.2 (1 - x)^5: (x1 x2)^-0.2 from ln x1 + ln x2
+    const double t = (1.0 - x1) * (1.0 - x2), t2 = t * t;
+    double F = 2.89 * exp(-0.2 * P.lnxmin * (u1 + u2)) * (t2 * t2 * t);
+#pragma unroll
+    for (int i = 0; i < N - 2; ++i) F *= g2;
+    if constexpr (M >= 3) {
+#pragma unroll
+      for (int i = 0; i < M - 3; ++i) F *= shat;
+    } else {
+      F /= shat;
+    }
+    K.wf = P.wk * F;  // wk = wconst (ln x_min)^2 phiconst / 2
+  }
+}
+
+// Colour ordering and helicity labels as sample_positions gives them, as an
+// array: perm[a] is the leg at position a.
 template <int N>
 __device__ __forceinline__ uint32_t sample_config(const EventParams &P, uint64_t ev, int (&perm)[N]) {
   constexpr int M = N - 2;
@@ -353,13 +475,6 @@ __device__ __forceinline__ double pow2_unit_inv(double rs) {
   return ldexp(1.0, -e);
 }
 
-// x 2^s by adding s to the exponent field: equal to ldexp(x, s) for a normal
-// nonzero x whose result is normal (the callers' factors are far inside the
-// double range), in two integer operations instead of FP64 work.
-__device__ __forceinline__ double scale_pow2(double x, int s) {
-  return __longlong_as_double(__double_as_longlong(x) + ((long long)s << 52));
-}
-
 // Exact sum of |m|^2 over the (n-1)! orderings and 2^n helicity labellings,
 // n = 4 and 5.  What bounds it is the FP64 pipe (1/64 of the FP32 rate), so
 // terms that are equal or zero are not evaluated: flipping every label
@@ -373,13 +488,14 @@ __device__ __forceinline__ double scale_pow2(double x, int s) {
 // bits, in FP32, the largest error of 3,000 events at n = 4 was 5e-7 (9e-7 with
 // four-component currents), of 600 at n = 5 2e-5 (4e-4).
 template <typename R, int N>
-__device__ __forceinline__ double summed_amp2(const double (&kk)[N][4], double inv_rs) {
+__device__ __forceinline__ double summed_amp2(const double (&k)[N - 2][4], int ex) {
   constexpr int L = N - 1;
   LCLeg<R> leg[L];  // leg 1 (the second incoming gluon) and the outgoing ones
   leg[0] = {R(0), R(0), R(0), R(0), R(0), R(0)};
 #pragma unroll
   for (int l = 1; l < L; ++l)
-    leg[l] = lc_leg<R>(kk[l + 1][0] * inv_rs, kk[l + 1][1] * inv_rs, kk[l + 1][2] * inv_rs, kk[l + 1][3] * inv_rs);
+    leg[l] = lc_leg<R>(scale_pow2_z(k[l - 1][0], -ex), scale_pow2_z(k[l - 1][1], -ex), scale_pow2_z(k[l - 1][2], -ex),
+                       scale_pow2_z(k[l - 1][3], -ex));
   int perm[L];  // colour position -> leg - 1
 #pragma unroll
   for (int i = 0; i < L; ++i) perm[i] = i;
@@ -435,42 +551,26 @@ __device__ __forceinline__ EventResult event(const EventParams &P, uint64_t ev) 
   constexpr int M = N - 2;
   Kinematics<N> K;
   kinematics<N>(P, ev, K);
-  const double inv_rs = pow2_unit_inv(sqrt(K.shat));
+  const int ex = exponent_of(K.rs);
   double E;
   if constexpr (SUM) {
-    E = P.efac * summed_amp2<R, N>(K.kk, inv_rs);  // efac = 1 / 2^(n-2) in this mode
+    E = P.efac * summed_amp2<R, N>(K.k, ex);  // efac = 1 / 2^(n-2) in this mode
   } else {
+    double kk[N][4];
+    const double h = 0.5 * K.rs;
+    kk[0][0] = -h; kk[0][1] = 0.0; kk[0][2] = 0.0; kk[0][3] = -h;
+    kk[1][0] = -h; kk[1][1] = 0.0; kk[1][2] = 0.0; kk[1][3] = h;
+#pragma unroll
+    for (int i = 0; i < M; ++i)
+#pragma unroll
+      for (int m = 0; m < 4; ++m) kk[2 + i][m] = K.k[i][m];
     int perm[N];
     const uint32_t hel = sample_config<N>(P, ev, perm);
-    E = P.efac * ordered_amp2<R, N>(K.kk, inv_rs, perm, hel);
+    E = P.efac * ordered_amp2<R, N>(kk, pow2_unit_inv(K.rs), perm, hel);
   }
   // |m|^2 has mass dimension 8 - 2n: undo the momentum unit (exact)
-  const double u2 = inv_rs * inv_rs;
-#pragma unroll
-  for (int i = 0; i < N - 4; ++i) E *= u2;
-  EventResult r;
-  r.me2 = E;
-  r.ht = K.ht;
-  r.ptlead = K.ptlead;
-  r.rmin = K.rmin;
-  r.pass = K.pass;
-  r.w = 0.0;
-  if (K.pass) {
-    const double mu = P.mu_r_factor * K.ht;
-    const double as = P.alphas_mz / (1.0 + P.alphas_mz * P.b0 * (log(mu * mu) - P.ln_mz2));
-    const double g2 = 4.0 * 3.14159265358979323846 * as;
-    double gp = 1.0;
-#pragma unroll
-    for (int i = 0; i < N - 2; ++i) gp *= g2;
-    double sp = 1.0;
-#pragma unroll
-    for (int i = 0; i < M - 2; ++i) sp *= K.shat;
-    const double f1 = 1.7 * pow(K.x1, -0.2) * pow(1.0 - K.x1, 5.0);
-    const double f2 = 1.7 * pow(K.x2, -0.2) * pow(1.0 - K.x2, 5.0);
-    const double lum = P.lnxmin * P.lnxmin * f1 * f2;
-    r.w = P.wconst * lum / (2.0 * K.shat) * (P.phiconst * sp) * gp * E;
-  }
-  return r;
+  E *= scale_pow2(1.0, -2 * ex * (N - 4));
+  return {K.wf * E, E, K.ht, K.ptlead, K.rmin, K.pass};
 }
 
 }  // namespace tess

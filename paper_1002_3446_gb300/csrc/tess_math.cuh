@@ -27,11 +27,12 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
   return c;
 }
 
-// 52 random bits (26 from each word) -> (k + 1/2) 2^-52, exact in double and
-// strictly inside (0, 1).
+// 52 random bits k (26 from each word) -> (k + 1/2) 2^-52, exact in double and
+// strictly inside (0, 1): k as the fraction of a double in [1, 2), less 1 - 2^-53
+// (one FP64 operation; conversions run on the same 1/64-rate pipe).
 __device__ __forceinline__ double unit_from_words(uint32_t a, uint32_t b) {
-  const double hi = (double)(a >> 6), lo = (double)(b >> 6);
-  return (hi * 67108864.0 + lo + 0.5) * 0x1p-52;
+  const uint64_t k = ((uint64_t)(a >> 6) << 26) | (uint64_t)(b >> 6);
+  return __longlong_as_double((long long)(0x3ff0000000000000ull | k)) - 0x1.fffffffffffffp-1;
 }
 
 // Uniforms number 2*blk and 2*blk+1 of event `ev` in stream `seed`: one

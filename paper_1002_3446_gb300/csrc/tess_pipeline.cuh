@@ -82,48 +82,6 @@ __device__ __forceinline__ void load_eps(const R *p, size_t s, CV4<R> &v) {
   v.c[3].im = R(0);
 }
 
-template <typename R>
-__device__ __forceinline__ R r_exp(R x);
-template <>
-__device__ __forceinline__ float r_exp<float>(float x) { return expf(x); }
-template <>
-__device__ __forceinline__ double r_exp<double>(double x) { return exp(x); }
-
-template <typename R>
-__device__ __forceinline__ R r_log(R x);
-template <>
-__device__ __forceinline__ float r_log<float>(float x) { return logf(x); }
-template <>
-__device__ __forceinline__ double r_log<double>(double x) { return log(x); }
-
-template <typename R>
-__device__ __forceinline__ R r_atan2(R y, R x);
-template <>
-__device__ __forceinline__ float r_atan2<float>(float y, float x) { return atan2f(y, x); }
-template <>
-__device__ __forceinline__ double r_atan2<double>(double y, double x) { return atan2(y, x); }
-
-template <typename R>
-__device__ __forceinline__ void r_sincospi(R x, R *s, R *c);
-template <>
-__device__ __forceinline__ void r_sincospi<float>(float x, float *s, float *c) { sincospif(x, s, c); }
-template <>
-__device__ __forceinline__ void r_sincospi<double>(double x, double *s, double *c) { sincospi(x, s, c); }
-
-template <typename R>
-__device__ __forceinline__ R r_pow(R x, R y);
-template <>
-__device__ __forceinline__ float r_pow<float>(float x, float y) { return powf(x, y); }
-template <>
-__device__ __forceinline__ double r_pow<double>(double x, double y) { return pow(x, y); }
-
-// A uniform rounded to R, kept strictly below 1.
-template <typename R>
-__device__ __forceinline__ R r_unit(double u) {
-  R v = R(u);
-  return v < R(1) ? v : R(1) - R(1) / R(1 << 24);
-}
-
 // Random real polarisations (Sec. 3): cos and sin of the angle phi = 2 pi u of
 // every leg, from the draws after the colour-ordering draws (positions
 // 2 + 4m + 1 + (n - 2) + l of the event's draw layout).
@@ -235,169 +193,101 @@ __device__ __forceinline__ float grid_alphas(const EventParams &P, float ht) {
   return grid_blend(P.grid_as, kAsSegments, __fmul_rn(__fsub_rn(v, P.f_as_vlo), P.f_as_inv));
 }
 
-// K1, FP64 form: every step in double precision.
-template <int N, typename R, bool RP>
-__device__ __forceinline__ void kin_generic(const ChunkParams &C, const ChunkBuf<R> &B, int e) {
+// K1, FP64 form: every step in double precision (bounded by the FP64 pipe;
+// see kinematics for what stays off it).
+template <int N, bool RP>
+__device__ __forceinline__ void kin_fp64(const ChunkParams &C, const ChunkBuf<double> &B, int e) {
   constexpr int M = N - 2, L = N - 1;
+  using IR = InRows<L>;
   const EventParams &P = C.P;
   const uint64_t idx = C.chunk_first + (uint64_t)e;
   const uint64_t ev = P.first_event + idx;
+  Kinematics<N> K;
+  kinematics<N>(P, ev, K);
+  if (P.ht) P.ht[idx] = K.ht;
+  if (P.ptlead) P.ptlead[idx] = K.ptlead;
+  if (P.rmin) P.rmin[idx] = K.rmin;
+  if (P.pass) P.pass[idx] = (uint8_t)K.pass;
+  const int ex = exponent_of(K.rs);  // momentum unit 2^-ex
+  B.efac[e] = scale_pow2(P.efac, -2 * ex * (N - 4));
+  B.wfac[e] = K.wf;
+  B.pass[e] = (uint8_t)K.pass;
+  if (B.hval) B.hval[e] = P.hist_obs == 0 ? K.ptlead : (P.hist_obs == 1 ? K.ht : K.rmin);
 
-  // ---- x1, x2 (uniform in ln x)
-  const double2 ux = uniform_pair(P.seed, ev, 0);
-  const R x1 = r_exp<R>(R(ux.x) * R(P.lnxmin));
-  const R x2 = r_exp<R>(R(ux.y) * R(P.lnxmin));
-  const double shat = (double)x1 * (double)x2 * P.S;
-  const double rs = sqrt(shat);
-
-  // ---- Rambo: isotropic seeds in R, boost + rescale in FP64
-  double q[M][4];
-  double Q0 = 0.0, Q1 = 0.0, Q2 = 0.0, Q3 = 0.0;
+  // per leg: momentum in its unit, and the polarisation basis e1 = (ct cf, ct sf,
+  // -st), e2 = (-sf, cf, 0) of its physical direction (the beam-axis legs' ct
+  // rounded as the others', the same bits as polarisations gives)
+  double lk[N][4], e1[N][3], e2[N][2];
+  const double h = 0.5 * K.rs, hu = scale_pow2(h, -ex), ct0 = h * (1.0 / sqrt(h * h));
+  lk[0][0] = -hu; lk[0][1] = 0.0; lk[0][2] = 0.0; lk[0][3] = -hu;
+  lk[1][0] = -hu; lk[1][1] = 0.0; lk[1][2] = 0.0; lk[1][3] = hu;
+  e1[0][0] = ct0; e1[0][1] = 0.0; e1[0][2] = 0.0; e2[0][0] = 0.0; e2[0][1] = 1.0;   // physical +z
+  e1[1][0] = -ct0; e1[1][1] = 0.0; e1[1][2] = 0.0; e2[1][0] = 0.0; e2[1][1] = 1.0;  // physical -z
 #pragma unroll
   for (int i = 0; i < M; ++i) {
-    const double2 a = uniform_pair(P.seed, ev, 1 + 2 * i);
-    const double2 b = uniform_pair(P.seed, ev, 2 + 2 * i);
-    const R c = R(2) * r_unit<R>(a.x) - R(1);
-    const R s = sqrt(fmax(R(1) - c * c, R(0)));
-    R sn, cs;
-    r_sincospi<R>(R(2) * r_unit<R>(a.y), &sn, &cs);
-    const R q0 = -r_log<R>(r_unit<R>(b.x) * r_unit<R>(b.y));
-    q[i][0] = (double)q0;
-    q[i][1] = (double)(q0 * s * cs);
-    q[i][2] = (double)(q0 * s * sn);
-    q[i][3] = (double)(q0 * c);
-    Q0 += q[i][0];
-    Q1 += q[i][1];
-    Q2 += q[i][2];
-    Q3 += q[i][3];
-  }
-  const double Mq = sqrt(Q0 * Q0 - Q1 * Q1 - Q2 * Q2 - Q3 * Q3);
-  const double invM = 1.0 / Mq;
-  const double bx = -Q1 * invM, by = -Q2 * invM, bz = -Q3 * invM;
-  const double gam = Q0 * invM;
-  const double aa = 1.0 / (1.0 + gam);
-  const double xs = rs * invM;
-  double kk[N][4];
-  const double h = 0.5 * rs;
-  kk[0][0] = -h; kk[0][1] = 0.0; kk[0][2] = 0.0; kk[0][3] = -h;
-  kk[1][0] = -h; kk[1][1] = 0.0; kk[1][2] = 0.0; kk[1][3] = h;
-#pragma unroll
-  for (int i = 0; i < M; ++i) {
-    const double bq = bx * q[i][1] + by * q[i][2] + bz * q[i][3];
-    kk[2 + i][0] = xs * (gam * q[i][0] + bq);
-    const double f = aa * bq + q[i][0];
-    kk[2 + i][1] = xs * (q[i][1] + bx * f);
-    kk[2 + i][2] = xs * (q[i][2] + by * f);
-    kk[2 + i][3] = xs * (q[i][3] + bz * f);
-  }
-
-  // ---- cuts and observables (R), lab rapidity = eta + ln(x1/x2)/2
-  const R y = R(0.5) * r_log<R>(x1 / x2);
-  R eta[M], pt[M], px[M], py[M];
-  int pass = 1;
-  R sum = R(0), lead = R(0);
-#pragma unroll
-  for (int i = 0; i < M; ++i) {
-    px[i] = R(kk[2 + i][1]);
-    py[i] = R(kk[2 + i][2]);
-    const R pz = R(kk[2 + i][3]);
-    const R pt2 = px[i] * px[i] + py[i] * py[i];
-    const R pabs = sqrt(pt2 + pz * pz);
-    pt[i] = sqrt(pt2);
-    eta[i] = R(0.5) * r_log<R>((pabs + pz) / (pabs - pz)) + y;
-    sum += pt[i];
-    lead = fmax(lead, pt[i]);
-    pass &= (pt[i] > R(P.pt_min)) & (fabs(eta[i]) < R(P.eta_max));
-  }
-  R dr2min = R(1e30);
-#pragma unroll
-  for (int i = 0; i < M; ++i) {
-#pragma unroll
-    for (int j = i + 1; j < M; ++j) {
-      const R dphi = r_atan2<R>(fabs(px[i] * py[j] - py[i] * px[j]), px[i] * px[j] + py[i] * py[j]);
-      const R de = eta[i] - eta[j];
-      const R dr2 = de * de + dphi * dphi;
-      dr2min = fmin(dr2min, dr2);
-      pass &= (dr2 > R(P.dr2_min));
+    const double *k = K.k[i];
+    const double inv_p = 1.0 / sqrt(K.pt2[i] + k[3] * k[3]);
+    const double ct = k[3] * inv_p;
+    double cf = 1.0, sf = 0.0;
+    if (K.pt[i] > 0.0) {
+      const double inv_pt = 1.0 / K.pt[i];
+      cf = k[1] * inv_pt;
+      sf = k[2] * inv_pt;
     }
+    e1[2 + i][0] = ct * cf;
+    e1[2 + i][1] = ct * sf;
+    e1[2 + i][2] = -(K.pt[i] * inv_p);
+    e2[2 + i][0] = -sf;
+    e2[2 + i][1] = cf;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) lk[2 + i][m] = scale_pow2_z(k[m], -ex);
   }
-  const double ht = (double)sum, ptlead = (double)lead, rmin = (double)sqrt(dr2min);
-  if (P.ht) P.ht[idx] = ht;
-  if (P.ptlead) P.ptlead[idx] = ptlead;
-  if (P.rmin) P.rmin[idx] = rmin;
-  if (P.pass) P.pass[idx] = (uint8_t)pass;
-
-  // ---- weight factor (everything but the matrix element)
-  double wf = 0.0;
-  if (pass) {
-    const R mu = R(P.mu_r_factor) * sum;
-    const R as = R(P.alphas_mz) / (R(1) + R(P.alphas_mz) * R(P.b0) * (r_log<R>(mu * mu) - R(P.ln_mz2)));
-    const double g2 = 4.0 * 3.14159265358979323846 * (double)as;
-    double gp = 1.0;
-#pragma unroll
-    for (int i = 0; i < N - 2; ++i) gp *= g2;
-    double sp = 1.0;
-#pragma unroll
-    for (int i = 0; i < M - 2; ++i) sp *= shat;
-    const R f1 = R(1.7) * r_pow<R>(x1, R(-0.2)) * r_pow<R>(R(1) - x1, R(5));
-    const R f2 = R(1.7) * r_pow<R>(x2, R(-0.2)) * r_pow<R>(R(1) - x2, R(5));
-    const double lum = P.lnxmin * P.lnxmin * (double)f1 * (double)f2;
-    wf = P.wconst * lum / (2.0 * shat) * (P.phiconst * sp) * gp;
-  }
-  const double inv_rs = pow2_unit_inv(rs);
-  double ef = P.efac;
-  const double u2 = inv_rs * inv_rs;
-#pragma unroll
-  for (int i = 0; i < N - 4; ++i) ef *= u2;
-  B.efac[e] = ef;
-  B.wfac[e] = wf;
-  B.pass[e] = (uint8_t)pass;
-  if (B.hval) B.hval[e] = P.hist_obs == 0 ? ptlead : (P.hist_obs == 1 ? ht : rmin);
-
-  // ---- colour ordering, then sampled helicities or random real
-  // polarisations (FP64 construction)
+  // ---- colour ordering, then sampled helicities or random real polarisations
   int perm[N];
   const uint32_t hel = sample_config<N>(P, ev, perm);
   double cphi[N], sphi[N];
   if constexpr (RP) polarisation_angles<N, double>(P, ev, cphi, sphi);
-  double kp[N][4];
-  int legp[N];
-  gather_positions<N>(kk, perm, kp, legp);
-  const int cap = B.cap;
+  const size_t cap = (size_t)B.cap;
+  const double r2 = 0.70710678118654752440;
 #pragma unroll
   for (int a = 0; a < N; ++a) {
-    const double sg = legp[a] < 2 ? -1.0 : 1.0;
-    CV4<double> ep, em;
-    polarisations<double>(sg * kp[a][1], sg * kp[a][2], sg * kp[a][3], ep, em);
-    using IR = InRows<L>;
-    R *o = B.in + (size_t)(a == 0 ? IR::eps0 : IR::eps(a - 1)) * cap + e;
-    if (a > 0) {
-      R *ok = B.in + (size_t)IR::k(a - 1) * cap + e;
+    // the leg at colour position a (leg 0 stays at position 0)
+    double k[4], v[5], c = 0.0, s = 0.0;
+    const int want = a == 0 ? 0 : perm[a];
+    const int l0 = a == 0 ? 0 : 1;
 #pragma unroll
-      for (int m = 0; m < 4; ++m) ok[(size_t)m * cap] = R(kp[a][m] * inv_rs);
+    for (int l = l0; l < (a == 0 ? 1 : N); ++l) {
+      const bool hit = l == l0 || want == l;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) k[m] = hit ? lk[l][m] : k[m];
+#pragma unroll
+      for (int m = 0; m < 3; ++m) v[m] = hit ? e1[l][m] : v[m];
+#pragma unroll
+      for (int m = 0; m < 2; ++m) v[3 + m] = hit ? e2[l][m] : v[3 + m];
+      if constexpr (RP) {
+        c = hit ? cphi[l] : c;
+        s = hit ? sphi[l] : s;
+      }
+    }
+    double *o = B.in + (size_t)(a == 0 ? IR::eps0 : IR::eps(a - 1)) * cap + e;
+    if (a > 0) {
+      double *ok = B.in + (size_t)IR::k(a - 1) * cap + e;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) ok[(size_t)m * cap] = k[m];
     }
     if constexpr (RP) {
-      // eps_+ = -(e1 + i e2)/sqrt2, so cos e1 + sin e2 = -sqrt2 (cos Re + sin Im) eps_+
-      double cl = 0.0, sl = 0.0;
-#pragma unroll
-      for (int l = 0; l < N; ++l)
-        if (legp[a] == l) {
-          cl = cphi[l];
-          sl = sphi[l];
-        }
-      const double r = -1.41421356237309504880;
-#pragma unroll
-      for (int m = 1; m < 4; ++m) o[(size_t)(m - 1) * cap] = R(r * (cl * ep.c[m].re + sl * ep.c[m].im));
-      o[(size_t)3 * cap] = R(0);
-      o[(size_t)4 * cap] = R(0);
+      o[0] = fma(c, v[0], s * v[3]);
+      o[cap] = fma(c, v[1], s * v[4]);
+      o[2 * cap] = c * v[2];
+      o[3 * cap] = 0.0;
+      o[4 * cap] = 0.0;
     } else {
-      const bool minus = (hel >> legp[a]) & 1u;
-      const CV4<double> &z = minus ? em : ep;
-      o[0] = R(z.c[1].re);
-      o[(size_t)cap] = R(z.c[2].re);
-      o[(size_t)2 * cap] = R(z.c[3].re);
-      o[(size_t)3 * cap] = R(z.c[1].im);
-      o[(size_t)4 * cap] = R(z.c[2].im);
+      const double sre = ((hel >> want) & 1u) ? r2 : -r2;  // eps_-+ = (+-e1 - i e2) / sqrt2
+      o[0] = sre * v[0];
+      o[cap] = sre * v[1];
+      o[2 * cap] = sre * v[2];
+      o[3 * cap] = -r2 * v[3];
+      o[4 * cap] = -r2 * v[4];
     }
   }
 }
@@ -950,7 +840,7 @@ __global__ void __launch_bounds__(kBlock) kin_kernel(ChunkParams C, ChunkBuf<R> 
     store_tile<N>(B, kin_tile);
   } else {
     if (e >= C.count) return;
-    kin_generic<N, R, RP>(C, B, e);
+    kin_fp64<N, RP>(C, B, e);
   }
 }
 
