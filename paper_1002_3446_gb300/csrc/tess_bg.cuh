@@ -281,12 +281,33 @@ __device__ __forceinline__ R bg_amplitude_real(const RV4<R> (&k)[L], const RV4<R
   return rdot_l<true, false>(e0, num);  // e0: leg 0's polarisation vector
 }
 
+// a.k (complex a, real k), LEAF: a is a single leg's polarisation vector
+template <bool LEAF, typename R>
+__device__ __forceinline__ Cx<R> mdot_k(const CV4<R> &a, const RV4<R> &k) {
+  if constexpr (LEAF)
+    return mdot_leaf(a, k);
+  else
+    return mdot(a, k);
+}
+
+template <bool LEAF, typename R>
+__device__ __forceinline__ void axpy_l(CV4<R> &acc, const Cx<R> &s, const CV4<R> &v) {
+  if constexpr (LEAF)
+    axpy_leaf(acc, s, v);
+  else
+    axpy(acc, s, v);
+}
+
 // ---------------------------------------------------------------------------
 // Loop form of the same recursion for large tables (FP64, and FP32 with
 // n >= 8): runtime loops over lengths, sets and splits, the table in
 // per-thread local memory indexed by tri(a, b).  Compiles in O(1) code size.
 // The caller fills the single-leg entries J[tri(a,a)] (polarisations) and
-// K[tri(a,a)] (momenta) in colour order, then calls run().
+// K[tri(a,a)] (momenta) in colour order, then calls run(), which doubles the
+// momenta (the brackets need 2 J.K; scaling by two is exact).  FP64 work bounds
+// it (the pipe runs at 1/64 of the FP32 rate), so the first and last trips of
+// the loops over splits and triples, whose parts are single legs, have code of
+// their own that leaves out the legs' exact zeros (the results keep their bits).
 // ---------------------------------------------------------------------------
 template <typename R, int L>
 struct BGLoop {
@@ -297,9 +318,44 @@ struct BGLoop {
 
   __device__ __forceinline__ static int tri(int a, int b) { return a * L - (a * (a - 1)) / 2 + (b - a); }
 
+  // split ([a..i], [i+1..b]); LL / LR: the part is a single leg (its S is zero)
+  template <bool LL, bool LR>
+  __device__ __forceinline__ void split(int a, int i, int b, CV4<R> &acc, Cx<R> &s) const {
+    const int l = tri(a, i), r = tri(i + 1, b);
+    const CV4<R> Jl = J[l], Jr = J[r];
+    const RV4<R> Kl = K[l], Kr = K[r];
+    const Cx<R> d = mdot_l<LL, LR>(Jl, Jr);
+    Cx<R> cr = mdot_k<LL>(Jl, Kr), cl = mdot_k<LR>(Jr, Kl);
+    if constexpr (!LL) cr = cx<R>(cr.re - S[l].re, cr.im - S[l].im);
+    if constexpr (!LR) cl = cx<R>(cl.re + S[r].re, cl.im + S[r].im);
+    axpy_l<LR>(acc, cr, Jr);
+    axpy_l<LL>(acc, cx<R>(-cl.re, -cl.im), Jl);
+    axpy(acc, cx<R>(R(0.5) * d.re, R(0.5) * d.im), rsub(Kl, Kr));
+    s.re += d.re;
+    s.im += d.im;
+  }
+
+  // triples ([a..i], [i+1..j], [j+1..b]) of one i; LA: [a..i] is a single leg
+  template <bool LA>
+  __device__ __forceinline__ void triples(int a, int i, int b, CV4<R> &trs) const {
+    const CV4<R> JA = J[tri(a, i)];
+    if (i + 1 == b - 1) {
+      axpy_leaf(trs, mdot_l<LA, true>(JA, J[tri(b, b)]), J[tri(i + 1, i + 1)]);
+      return;
+    }
+    axpy_leaf(trs, mdot_l<LA, false>(JA, J[tri(i + 2, b)]), J[tri(i + 1, i + 1)]);
+#pragma unroll 1
+    for (int j = i + 2; j < b - 1; ++j) axpy(trs, mdot_l<LA, false>(JA, J[tri(j + 1, b)]), J[tri(i + 1, j)]);
+    axpy(trs, mdot_l<LA, true>(JA, J[tri(b, b)]), J[tri(i + 1, b - 1)]);
+  }
+
   __device__ Cx<R> run(const CV4<R> &e0) {
 #pragma unroll 1
-    for (int a = 0; a < L; ++a) S[tri(a, a)] = cx<R>(R(0), R(0));
+    for (int a = 0; a < L; ++a) {
+      const int X = tri(a, a);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) K[X].v[m] *= R(2);
+    }
     CV4<R> num = cv_zero<R>();
 #pragma unroll 1
     for (int len = 2; len <= L; ++len) {
@@ -307,32 +363,21 @@ struct BGLoop {
       for (int a = 0; a + len - 1 < L; ++a) {
         const int b = a + len - 1;
         const int X = tri(a, b);
-        K[X] = radd(K[tri(a, b - 1)], K[tri(b, b)]);
+        const RV4<R> KX = radd(K[tri(a, b - 1)], K[tri(b, b)]);
+        K[X] = KX;
         CV4<R> acc = cv_zero<R>();
         CV4<R> trs = cv_zero<R>();
         Cx<R> s = cx<R>(R(0), R(0));
+        if (len == 2) {
+          split<true, true>(a, a, b, acc, s);
+        } else {
+          split<true, false>(a, a, b, acc, s);
 #pragma unroll 1
-        for (int i = a; i < b; ++i) {
-          const int l = tri(a, i), r = tri(i + 1, b);
-          const CV4<R> Jl = J[l], Jr = J[r];
-          const RV4<R> Kl = K[l], Kr = K[r];
-          const Cx<R> d = mdot(Jl, Jr);
-          const Cx<R> jlkr = mdot(Jl, Kr);
-          const Cx<R> krjl = mdot(Jr, Kl);
-          const Cx<R> Sl = S[l], Sr = S[r];
-          const Cx<R> cr = cx<R>(fma(R(2), jlkr.re, -Sl.re), fma(R(2), jlkr.im, -Sl.im));
-          const Cx<R> cl = cx<R>(fma(R(-2), krjl.re, -Sr.re), fma(R(-2), krjl.im, -Sr.im));
-          axpy(acc, cr, Jr);
-          axpy(acc, cl, Jl);
-          axpy(acc, d, rsub(Kl, Kr));
-          s.re += d.re;
-          s.im += d.im;
-        }
+          for (int i = a + 1; i < b - 1; ++i) split<false, false>(a, i, b, acc, s);
+          split<false, true>(a, b - 1, b, acc, s);
+          triples<true>(a, a, b, trs);
 #pragma unroll 1
-        for (int i = a; i + 1 < b; ++i) {
-          const CV4<R> JA = J[tri(a, i)];
-#pragma unroll 1
-          for (int j = i + 1; j < b; ++j) axpy(trs, mdot(JA, J[tri(j + 1, b)]), J[tri(i + 1, j)]);
+          for (int i = a + 1; i + 1 < b; ++i) triples<false>(a, i, b, trs);
         }
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
@@ -340,7 +385,7 @@ struct BGLoop {
           acc.c[m].im = fma(R(2), trs.c[m].im, acc.c[m].im);
         }
         if (len < L) {
-          const R inv = R(1) / mdot(K[X], K[X]);
+          const R inv = R(4) / mdot(KX, KX);
 #pragma unroll
           for (int m = 0; m < 4; ++m) {
             J[X].c[m].re = acc.c[m].re * inv;
@@ -351,6 +396,13 @@ struct BGLoop {
           num = acc;
         }
       }
+    }
+    // the single legs' momenta as the caller gave them (it may run again)
+#pragma unroll 1
+    for (int a = 0; a < L; ++a) {
+      const int X = tri(a, a);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) K[X].v[m] *= R(0.5);
     }
     return mdot(e0, num);
   }
