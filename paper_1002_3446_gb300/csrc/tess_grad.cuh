@@ -626,10 +626,14 @@ __global__ void __launch_bounds__(kBlock) grad_kernel(GradParams G) {
   bg.forward();
   const Cx<R> mamp = mdot(e0, bg.num);
   CV4<R> ge0;
-  bg.adjoint(e0, cx<R>(R(2) * mamp.re, R(2) * mamp.im), ge0);
+  // weights alone (the forward pass of the autograd function): no reverse sweep
+  const bool sweep = G.dw_du || G.dw_dk || G.dw_dlnmu;
+  if (sweep) bg.adjoint(e0, cx<R>(R(2) * mamp.re, R(2) * mamp.im), ge0);
   const double f = (double)mamp.re * (double)mamp.re + (double)mamp.im * (double)mamp.im;
   grad_outputs<N, R, R>(G, e, K, hel, f, [&](int a, double(&g4)[4], CV4<R> &ge) {
-    if (a == 0) {
+    if (!sweep) {
+      ge = cv_zero<R>();
+    } else if (a == 0) {
       ge = ge0;
     } else {
       const int X = BGAdjoint<R, L>::tri(a - 1, a - 1);

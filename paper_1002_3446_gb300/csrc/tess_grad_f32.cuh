@@ -249,6 +249,36 @@ __device__ __forceinline__ void grad_amp_input_f32(const GradKinF<N> &K, uint32_
   for (int m = 0; m < 4; ++m) k.v[m] = K.kp[a][m] * c;
 }
 
+// Factors of the weight w = wfac(x, H_T) E(k), E = efac' f, of an event that
+// passes the cuts, as the kinematics kernel forms them: wfac = wk F 2^(2 ex
+// (m-3)) with F the FP32 product of PDFs, couplings and the scaled s_hat.
+// Returns wfac efac' (0 if it fails) and alpha_s.
+template <int N>
+__device__ __forceinline__ double grad_weight_factor(const EventParams &P, const GradKinF<N> &K, float &as) {
+  constexpr int M = N - 2;
+  as = 0.f;
+  if (!K.pass) return 0.0;
+  const float c = ldexpf(1.f, -K.ex);
+  const float mu = P.f_mu_r_factor * K.ht;
+  as = P.f_alphas_mz / (1.f + P.f_asb0 * (logf(mu * mu) - P.f_ln_mz2));
+  const float g2 = 4.f * 3.14159265358979323846f * as;
+  const float t1 = 1.f - K.x1, t2 = 1.f - K.x2;
+  const float t1s = t1 * t1, t2s = t2 * t2;
+  float F = 2.89f * expf(-0.2f * P.f_lnxmin * (K.ux1 + K.ux2)) * (t1s * t1s * t1) * (t2s * t2s * t2);
+#pragma unroll
+  for (int i = 0; i < N - 2; ++i) F *= g2;
+  const float sp = K.shat_hi * c * c;
+  if (M >= 3) {
+#pragma unroll
+    for (int i = 0; i < M - 3; ++i) F *= sp;
+  } else {
+    F /= sp;
+  }
+  if (!(F > 0.f)) return 0.0;
+  const double wf = scale_pow2(P.wk * f64_of_f32_scaled(F, 0), 2 * K.ex * (M - 3));
+  return wf * scale_pow2(P.efac, -2 * K.ex * (N - 4));
+}
+
 // Weights and gradients of event e from its kinematics and f = |m|^2 (in the
 // unit c); get(a, g4, ge) gives df/dk' of colour position a (k' = c k; zero
 // for position 0) and df/d eps (g(z) = df/dRe z + i df/dIm z).  Same
@@ -262,33 +292,9 @@ __device__ __forceinline__ void grad_outputs_f32(const GradParams &G, uint64_t e
   const float lnx = P.f_lnxmin;
   const float c = ldexpf(1.f, -K.ex);
 
-  // weight factors as the kinematics kernel forms them: wfac = wk F 2^(2 ex
-  // (m-3)) with F the FP32 product of PDFs, couplings and the scaled s_hat
-  double w = 0.0, A = 0.0;
-  float as = 0.f;
-  if (K.pass) {
-    const float mu = P.f_mu_r_factor * K.ht;
-    as = P.f_alphas_mz / (1.f + P.f_asb0 * (logf(mu * mu) - P.f_ln_mz2));
-    const float g2 = 4.f * 3.14159265358979323846f * as;
-    const float t1 = 1.f - K.x1, t2 = 1.f - K.x2;
-    const float t1s = t1 * t1, t2s = t2 * t2;
-    float F = 2.89f * expf(-0.2f * lnx * (K.ux1 + K.ux2)) * (t1s * t1s * t1) * (t2s * t2s * t2);
-#pragma unroll
-    for (int i = 0; i < N - 2; ++i) F *= g2;
-    const float sp = K.shat_hi * c * c;
-    if (M >= 3) {
-#pragma unroll
-      for (int i = 0; i < M - 3; ++i) F *= sp;
-    } else {
-      F /= sp;
-    }
-    if (F > 0.f) {
-      const double wf = scale_pow2(P.wk * f64_of_f32_scaled(F, 0), 2 * K.ex * (M - 3));
-      const double Aw = wf * scale_pow2(P.efac, -2 * K.ex * (N - 4));
-      w = Aw * f;
-      A = (G.dL_dw ? G.dL_dw[e] : 1.0) * Aw;
-    }
-  }
+  float as;
+  const double Aw = grad_weight_factor<N>(P, K, as);
+  const double w = Aw == 0.0 ? 0.0 : Aw * f, A = (G.dL_dw ? G.dL_dw[e] : 1.0) * Aw;
   if (G.w) G.w[e] = w;
   double *gu = G.dw_du ? G.dw_du + e * NU : nullptr;
   double *gkout = G.dw_dk ? G.dw_dk + e * N * 4 : nullptr;
