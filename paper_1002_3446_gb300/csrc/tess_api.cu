@@ -1045,6 +1045,7 @@ int tess_gradients(tess_ctx *ctx, const tess_process *proc, uint64_t n_events, c
   G.dw_dlnmu = dw_dlnmu;
   G.n_events = n_events;
   G.chunk_bytes = ctx->chunk_bytes;
+  G.sm_count = ctx->sm_count;
   const int n = proc->n_gluons;
   const bool fp64 = proc->precision == TESS_FP64;
   size_t need = 0;

@@ -217,38 +217,65 @@ __device__ void pull_set(const float4 *J4, const float4 *G4, const float4 *P4, c
 // above, grad_amp_kernel stopped after the recursion).  The eps gradients keep the five
 // components the polarisation adjoint reads (Re x, y, z; Im x, y).
 // ---------------------------------------------------------------------------
+// Events that fail the cuts have w = 0 and zero gradients, so only the others
+// (a tenth at n = 8 with the default cuts) go past G1: it gives each a column
+// of the chunk (in no particular order: every output has a place of its own,
+// and no event's arithmetic depends on its column), and zeroes the chunk's
+// outputs.
 struct GradChunk {
   float *in;  // [InRows<L>::rows][cap]
   float *gr;  // [InRows<L>::rows][cap]: df/dk (4) and df/deps (5) per position 1..L, then df/deps_0
-  double *f;  // [cap] |m|^2
+  double *f;  // [cap] |m|^2 (weights alone: the weight factor)
+  int *orig;  // [cap] event of a column (index within the chunk)
+  int *n;     // [1] columns in use (zeroed before G1)
   int cap;
 };
+
+// Zeroes the block's events of an output of `per` doubles an event.
+__device__ __forceinline__ void grad_zero(double *out, uint64_t first, int count, int per) {
+  if (!out) return;
+  const int e0 = blockIdx.x * kBlock, ne = min(kBlock, count - e0);
+  double *o = out + (first + (uint64_t)e0) * per;
+  for (int i = threadIdx.x; i < ne * per; i += kBlock) o[i] = 0.0;
+}
 
 // WONLY: B.f receives the weight factor.
 template <int N, bool WONLY>
 __global__ void __launch_bounds__(kBlock) grad_in_kernel(GradParams G, uint64_t first, int count, GradChunk B) {
   constexpr int M = N - 2, L = N - 1, NU = 2 + 4 * M;
   const int e = blockIdx.x * kBlock + threadIdx.x;
-  if (e >= count) return;
-  const uint64_t ev = first + (uint64_t)e;
+  const uint64_t ev = first + (uint64_t)min(e, count - 1);
   GradKinF<N> K;
   grad_kin_f32<N>(G.P, G.u + ev * NU, G.order + ev * N, K);
+  const bool keep = e < count && K.pass;
+  __shared__ int base[kBlock / 32];
+  const unsigned m = __ballot_sync(0xffffffffu, keep);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane == 0) base[warp] = m ? atomicAdd(B.n, __popc(m)) : 0;
+  grad_zero(G.w, first, count, 1);
+  grad_zero(G.dw_dlnmu, first, count, 1);
+  grad_zero(G.dw_du, first, count, NU);
+  grad_zero(G.dw_dk, first, count, 4 * N);
+  __syncwarp();
+  if (!keep) return;
+  const int c = base[warp] + __popc(m & ((1u << lane) - 1u));  // its column
+  B.orig[c] = e;
   const uint32_t hel = G.hel[ev];
   const size_t cap = (size_t)B.cap;
   if constexpr (WONLY) {
     float as;
-    B.f[e] = grad_weight_factor<N>(G.P, K, as);
+    B.f[c] = grad_weight_factor<N>(G.P, K, as);
   }
 #pragma unroll
   for (int a = 0; a <= L; ++a) {
     RV4<float> k;
     CV4<float> eps;
     grad_amp_input_f32<N>(K, hel, a, k, eps);
-    float *o = B.in + (size_t)(a == 0 ? InRows<L>::eps0 : InRows<L>::eps(a - 1)) * cap + e;
+    float *o = B.in + (size_t)(a == 0 ? InRows<L>::eps0 : InRows<L>::eps(a - 1)) * cap + c;
     if (a > 0) {
-      float *ok = B.in + (size_t)InRows<L>::k(a - 1) * cap + e;
+      float *ok = B.in + (size_t)InRows<L>::k(a - 1) * cap + c;
 #pragma unroll
-      for (int m = 0; m < 4; ++m) ok[m * cap] = k.v[m];
+      for (int q = 0; q < 4; ++q) ok[q * cap] = k.v[q];
     }
     o[0] = eps.c[1].re;
     o[cap] = eps.c[2].re;
@@ -266,13 +293,14 @@ __device__ __forceinline__ double grad_weight(double factor, const Cx<float> &m)
 
 // Weights alone, n <= 8: thread per event, the current table in registers
 // (bg_amplitude).  The forward call of the autograd function at
-// n = 8 and 2^18 events: 184 us, 947 with the reverse sweep.
+// n = 8 and 2^18 events: 947 us with the reverse sweep, 184 without it, 90 with
+// the events that fail the cuts left out (27 of them here).
 template <int N>
 __global__ void __launch_bounds__(kBlock, N <= 5 ? 4 : (N == 6 ? 3 : 2))
-    grad_weight_kernel(int count, GradChunk B, double *__restrict__ w) {
+    grad_weight_kernel(GradChunk B, double *__restrict__ w) {
   constexpr int L = N - 1;
   const int e = blockIdx.x * kBlock + threadIdx.x;
-  if (e >= count) return;
+  if (e >= *B.n) return;
   const size_t cap = (size_t)B.cap;
   RV4<float> k[L];
   CV4<float> ev[L], e0;
@@ -282,12 +310,12 @@ __global__ void __launch_bounds__(kBlock, N <= 5 ? 4 : (N == 6 ? 3 : 2))
     load_eps(B.in + (size_t)InRows<L>::eps(a) * cap + e, cap, ev[a]);
   }
   load_eps(B.in + (size_t)InRows<L>::eps0 * cap + e, cap, e0);
-  w[e] = grad_weight(B.f[e], bg_amplitude<float, L>(k, ev, e0));
+  w[B.orig[e]] = grad_weight(B.f[e], bg_amplitude<float, L>(k, ev, e0));
 }
 
 // WONLY: ends with the weights w (B.f holds the factors).
 template <int N, int NEV, int LN, bool WONLY>
-__global__ void __launch_bounds__(LN * NEV) grad_amp_kernel(int count, GradChunk B, double *__restrict__ w) {
+__global__ void __launch_bounds__(LN * NEV) grad_amp_kernel(GradChunk B, double *__restrict__ w) {
   constexpr int L = N - 1;
   using PS = GradPairSmem<L, NEV, LN>;
   static_assert(LN >= 2 && LN - 1 <= PS::T, "the lanes' partial top sums use adjoint-table slots 0 .. LN-2");
@@ -297,177 +325,181 @@ __global__ void __launch_bounds__(LN * NEV) grad_amp_kernel(int count, GradChunk
   float2 *S2 = (float2 *)(smem_ga + PS::s_off), *gS2 = (float2 *)(smem_ga + PS::gs_off);
   const int lane = threadIdx.x / NEV, g = threadIdx.x % NEV;
   float4 *GP4 = (float4 *)(smem_ga + PS::gp_off) + (size_t)lane * (L + 1) * NEV;
-  const int e = blockIdx.x * NEV + g;
-  const bool live = e < count;
+  const int n = *B.n;
   const size_t cap = (size_t)B.cap;
-  if (live) {
-    if (lane == 0) {  // momenta -> prefix sums, eps_0
-      RV4<float> p = {{0.f, 0.f, 0.f, 0.f}};
-      P4[g] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
-      for (int a = 0; a < L; ++a) {
-        RV4<float> k;
-        load_k(B.in + (size_t)InRows<L>::k(a) * cap + e, cap, k);
-        p = radd(p, k);
-        P4[(a + 1) * NEV + g] = make_float4(p.v[0], p.v[1], p.v[2], p.v[3]);
-      }
-      CV4<float> e0;
-      load_eps(B.in + (size_t)InRows<L>::eps0 * cap + e, cap, e0);
-      E4[g] = make_float4(e0.c[0].re, e0.c[0].im, e0.c[1].re, e0.c[1].im);
-      E4[NEV + g] = make_float4(e0.c[2].re, e0.c[2].im, e0.c[3].re, e0.c[3].im);
-    } else {  // single-leg currents, shared by the other lanes
-#pragma unroll 1
-      for (int a = lane - 1; a < L; a += LN - 1) {
-        CV4<float> ea;
-        load_eps(B.in + (size_t)InRows<L>::eps(a) * cap + e, cap, ea);
-        const int X = pair_tri<L>(a, a);
-        st_cv4<NEV>(J4, X, g, ea);
-        S2[X * NEV + g] = make_float2(0.f, 0.f);
-      }
-    }
-  }
-#pragma unroll 1
-  for (int i = 0; i <= L; ++i) GP4[i * NEV + g] = make_float4(0.f, 0.f, 0.f, 0.f);
-  __syncthreads();
-  PairView<NEV> V;
-  V.J4 = J4;
-  V.P4 = P4;
-  V.E4 = E4;
-  V.S2 = S2;
-  V.g = g;
-#pragma unroll 1
-  for (int len = 2; len < L; ++len) {
+  for (int tile = blockIdx.x; tile * NEV < n; tile += gridDim.x) {  // uniform per block
+    const int e = tile * NEV + g;
+    const bool live = e < n;
     if (live) {
+      if (lane == 0) {  // momenta -> prefix sums, eps_0
+        RV4<float> p = {{0.f, 0.f, 0.f, 0.f}};
+        P4[g] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
-      for (int a = lane; a + len - 1 < L; a += LN) {
-        const int b = a + len - 1;
-        CV4<float> acc;
-        Cx<float> s;
-        pair_sums<L, NEV>(V, a, b, 0, 1, acc, s);
-        const RV4<float> Kab = rsub(V.P(b + 1), V.P(a));
-        const float inv = 1.f / mdot(Kab, Kab);
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-          acc.c[m].re *= inv;
-          acc.c[m].im *= inv;
+        for (int a = 0; a < L; ++a) {
+          RV4<float> k;
+          load_k(B.in + (size_t)InRows<L>::k(a) * cap + e, cap, k);
+          p = radd(p, k);
+          P4[(a + 1) * NEV + g] = make_float4(p.v[0], p.v[1], p.v[2], p.v[3]);
         }
-        const int X = pair_tri<L>(a, b);
-        V.setJ(X, acc);
-        S2[X * NEV + g] = make_float2(s.re, s.im);
+        CV4<float> e0;
+        load_eps(B.in + (size_t)InRows<L>::eps0 * cap + e, cap, e0);
+        E4[g] = make_float4(e0.c[0].re, e0.c[0].im, e0.c[1].re, e0.c[1].im);
+        E4[NEV + g] = make_float4(e0.c[2].re, e0.c[2].im, e0.c[3].re, e0.c[3].im);
+      } else {  // single-leg currents, shared by the other lanes
+#pragma unroll 1
+        for (int a = lane - 1; a < L; a += LN - 1) {
+          CV4<float> ea;
+          load_eps(B.in + (size_t)InRows<L>::eps(a) * cap + e, cap, ea);
+          const int X = pair_tri<L>(a, a);
+          st_cv4<NEV>(J4, X, g, ea);
+          S2[X * NEV + g] = make_float2(0.f, 0.f);
+        }
       }
     }
+#pragma unroll 1
+    for (int i = 0; i <= L; ++i) GP4[i * NEV + g] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
-  }
-  const int top = pair_tri<L>(0, L - 1);
-  CV4<float> num = cv_zero<float>();
-  if (live) {
-    Cx<float> s;
-    pair_sums<L, NEV>(V, 0, L - 1, lane, LN, num, s);
-    // the adjoint table is free until the sweep: scratch for the partial sums
-    if (lane > 0) st_cv4<NEV>(G4, lane - 1, g, num);
-  }
-  __syncthreads();
-  if (live && lane == 0) {
+    PairView<NEV> V;
+    V.J4 = J4;
+    V.P4 = P4;
+    V.E4 = E4;
+    V.S2 = S2;
+    V.g = g;
 #pragma unroll 1
-    for (int j = 1; j < LN; ++j) {
-      const CV4<float> other = ld_cv4<NEV>(G4, j - 1, g);
-#pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        num.c[m].re += other.c[m].re;
-        num.c[m].im += other.c[m].im;
-      }
-    }
-    const float4 u0 = E4[g], v0 = E4[NEV + g];
-    CV4<float> e0;
-    e0.c[0] = cx<float>(u0.x, u0.y);
-    e0.c[1] = cx<float>(u0.z, u0.w);
-    e0.c[2] = cx<float>(v0.x, v0.y);
-    e0.c[3] = cx<float>(v0.z, v0.w);
-    const Cx<float> mamp = mdot(e0, num);
-    if constexpr (WONLY) {
-      w[e] = grad_weight(B.f[e], mamp);
-      return;
-    }
-    B.f[e] = (double)mamp.re * (double)mamp.re + (double)mamp.im * (double)mamp.im;
-    const Cx<float> gm = cx<float>(2.f * mamp.re, 2.f * mamp.im);
-    CV4<float> ge0 = cv_zero<float>(), gtop = cv_zero<float>();
-    add_eta_conj(ge0, num, gm);
-    add_eta_conj(gtop, e0, gm);
-    st_cv4<NEV>(G4, top, g, gtop);
-    gS2[top * NEV + g] = make_float2(0.f, 0.f);
-    float *o = B.gr + (size_t)InRows<L>::eps0 * cap + e;
-    o[0] = ge0.c[1].re;
-    o[cap] = ge0.c[2].re;
-    o[2 * cap] = ge0.c[3].re;
-    o[3 * cap] = ge0.c[1].im;
-    o[4 * cap] = ge0.c[2].im;
-  }
-  if constexpr (WONLY) return;
-  __syncthreads();
+    for (int len = 2; len < L; ++len) {
+      if (live) {
 #pragma unroll 1
-  for (int len = L - 1; len >= 1; --len) {
-    if (live) {
-#pragma unroll 1
-      for (int c = lane; c + len - 1 < L; c += LN) {
-        const int d = c + len - 1, Y = pair_tri<L>(c, d);
-        CV4<float> GJ;
-        Cx<float> GS;
-        RV4<float> GK;
-        pull_set<L, NEV>(J4, G4, P4, S2, gS2, g, c, d, GJ, GS, GK);
-        if (len >= 2) {
-          const RV4<float> KY = rsub(rv4(P4[(d + 1) * NEV + g]), rv4(P4[c * NEV + g]));
-          const float inv = 1.f / mdot(KY, KY);
-          const Cx<float> cj = conj_dot4(V.J(Y), GJ);
-          const float gk2 = -2.f * cj.re * inv;
+        for (int a = lane; a + len - 1 < L; a += LN) {
+          const int b = a + len - 1;
+          CV4<float> acc;
+          Cx<float> s;
+          pair_sums<L, NEV>(V, a, b, 0, 1, acc, s);
+          const RV4<float> Kab = rsub(V.P(b + 1), V.P(a));
+          const float inv = 1.f / mdot(Kab, Kab);
 #pragma unroll
           for (int m = 0; m < 4; ++m) {
-            GK.v[m] = fmaf(gk2 * eta_of(m), KY.v[m], GK.v[m]);
-            GJ.c[m].re *= inv;
-            GJ.c[m].im *= inv;
+            acc.c[m].re *= inv;
+            acc.c[m].im *= inv;
           }
-          gS2[Y * NEV + g] = make_float2(GS.re, GS.im);
-          st_cv4<NEV>(G4, Y, g, GJ);
-        } else {  // a single leg: df/deps of position c + 1
-          float *o = B.gr + (size_t)InRows<L>::eps(c) * cap + e;
-          o[0] = GJ.c[1].re;
-          o[cap] = GJ.c[2].re;
-          o[2 * cap] = GJ.c[3].re;
-          o[3 * cap] = GJ.c[1].im;
-          o[4 * cap] = GJ.c[2].im;
+          const int X = pair_tri<L>(a, b);
+          V.setJ(X, acc);
+          S2[X * NEV + g] = make_float2(s.re, s.im);
         }
-        float4 hi = GP4[(d + 1) * NEV + g], lo = GP4[c * NEV + g];
-        GP4[(d + 1) * NEV + g] = make_float4(hi.x + GK.v[0], hi.y + GK.v[1], hi.z + GK.v[2], hi.w + GK.v[3]);
-        GP4[c * NEV + g] = make_float4(lo.x - GK.v[0], lo.y - GK.v[1], lo.z - GK.v[2], lo.w - GK.v[3]);
+      }
+      __syncthreads();
+    }
+    const int top = pair_tri<L>(0, L - 1);
+    CV4<float> num = cv_zero<float>();
+    if (live) {
+      Cx<float> s;
+      pair_sums<L, NEV>(V, 0, L - 1, lane, LN, num, s);
+      // the adjoint table is free until the sweep: scratch for the partial sums
+      if (lane > 0) st_cv4<NEV>(G4, lane - 1, g, num);
+    }
+    __syncthreads();
+    if (live && lane == 0) {
+#pragma unroll 1
+      for (int j = 1; j < LN; ++j) {
+        const CV4<float> other = ld_cv4<NEV>(G4, j - 1, g);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          num.c[m].re += other.c[m].re;
+          num.c[m].im += other.c[m].im;
+        }
+      }
+      const float4 u0 = E4[g], v0 = E4[NEV + g];
+      CV4<float> e0;
+      e0.c[0] = cx<float>(u0.x, u0.y);
+      e0.c[1] = cx<float>(u0.z, u0.w);
+      e0.c[2] = cx<float>(v0.x, v0.y);
+      e0.c[3] = cx<float>(v0.z, v0.w);
+      const Cx<float> mamp = mdot(e0, num);
+      if constexpr (WONLY) {
+        w[B.orig[e]] = grad_weight(B.f[e], mamp);
+      } else {
+        B.f[e] = (double)mamp.re * (double)mamp.re + (double)mamp.im * (double)mamp.im;
+        const Cx<float> gm = cx<float>(2.f * mamp.re, 2.f * mamp.im);
+        CV4<float> ge0 = cv_zero<float>(), gtop = cv_zero<float>();
+        add_eta_conj(ge0, num, gm);
+        add_eta_conj(gtop, e0, gm);
+        st_cv4<NEV>(G4, top, g, gtop);
+        gS2[top * NEV + g] = make_float2(0.f, 0.f);
+        float *o = B.gr + (size_t)InRows<L>::eps0 * cap + e;
+        o[0] = ge0.c[1].re;
+        o[cap] = ge0.c[2].re;
+        o[2 * cap] = ge0.c[3].re;
+        o[3 * cap] = ge0.c[1].im;
+        o[4 * cap] = ge0.c[2].im;
       }
     }
     __syncthreads();
-  }
-  if (live && lane == 0) {  // df/dk of BG leg t = sum over i > t of every lane's prefix rows
-    const float4 *GPa = (const float4 *)(smem_ga + PS::gp_off);
-    RV4<float> acc = {{0.f, 0.f, 0.f, 0.f}};
+    if constexpr (WONLY) continue;
 #pragma unroll 1
-    for (int t = L - 1; t >= 0; --t) {
+    for (int len = L - 1; len >= 1; --len) {
+      if (live) {
+#pragma unroll 1
+        for (int c = lane; c + len - 1 < L; c += LN) {
+          const int d = c + len - 1, Y = pair_tri<L>(c, d);
+          CV4<float> GJ;
+          Cx<float> GS;
+          RV4<float> GK;
+          pull_set<L, NEV>(J4, G4, P4, S2, gS2, g, c, d, GJ, GS, GK);
+          if (len >= 2) {
+            const RV4<float> KY = rsub(rv4(P4[(d + 1) * NEV + g]), rv4(P4[c * NEV + g]));
+            const float inv = 1.f / mdot(KY, KY);
+            const Cx<float> cj = conj_dot4(V.J(Y), GJ);
+            const float gk2 = -2.f * cj.re * inv;
 #pragma unroll
-      for (int j = 0; j < LN; ++j) {
-        const float4 a0 = GPa[((size_t)j * (L + 1) + t + 1) * NEV + g];
-        acc.v[0] += a0.x;
-        acc.v[1] += a0.y;
-        acc.v[2] += a0.z;
-        acc.v[3] += a0.w;
+            for (int m = 0; m < 4; ++m) {
+              GK.v[m] = fmaf(gk2 * eta_of(m), KY.v[m], GK.v[m]);
+              GJ.c[m].re *= inv;
+              GJ.c[m].im *= inv;
+            }
+            gS2[Y * NEV + g] = make_float2(GS.re, GS.im);
+            st_cv4<NEV>(G4, Y, g, GJ);
+          } else {  // a single leg: df/deps of position c + 1
+            float *o = B.gr + (size_t)InRows<L>::eps(c) * cap + e;
+            o[0] = GJ.c[1].re;
+            o[cap] = GJ.c[2].re;
+            o[2 * cap] = GJ.c[3].re;
+            o[3 * cap] = GJ.c[1].im;
+            o[4 * cap] = GJ.c[2].im;
+          }
+          float4 hi = GP4[(d + 1) * NEV + g], lo = GP4[c * NEV + g];
+          GP4[(d + 1) * NEV + g] = make_float4(hi.x + GK.v[0], hi.y + GK.v[1], hi.z + GK.v[2], hi.w + GK.v[3]);
+          GP4[c * NEV + g] = make_float4(lo.x - GK.v[0], lo.y - GK.v[1], lo.z - GK.v[2], lo.w - GK.v[3]);
+        }
       }
-      float *ok = B.gr + (size_t)InRows<L>::k(t) * cap + e;
-#pragma unroll
-      for (int m = 0; m < 4; ++m) ok[m * cap] = acc.v[m];
+      __syncthreads();
     }
+    if (live && lane == 0) {  // df/dk of BG leg t = sum over i > t of every lane's prefix rows
+      const float4 *GPa = (const float4 *)(smem_ga + PS::gp_off);
+      RV4<float> acc = {{0.f, 0.f, 0.f, 0.f}};
+#pragma unroll 1
+      for (int t = L - 1; t >= 0; --t) {
+#pragma unroll
+        for (int j = 0; j < LN; ++j) {
+          const float4 a0 = GPa[((size_t)j * (L + 1) + t + 1) * NEV + g];
+          acc.v[0] += a0.x;
+          acc.v[1] += a0.y;
+          acc.v[2] += a0.z;
+          acc.v[3] += a0.w;
+        }
+        float *ok = B.gr + (size_t)InRows<L>::k(t) * cap + e;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) ok[m * cap] = acc.v[m];
+      }
+    }
+    __syncthreads();  // the tables are read until here, and filled again by the next tile
   }
 }
 
 template <int N>
-__global__ void __launch_bounds__(kBlock) grad_out_kernel(GradParams G, uint64_t first, int count, GradChunk B) {
+__global__ void __launch_bounds__(kBlock) grad_out_kernel(GradParams G, uint64_t first, GradChunk B) {
   constexpr int M = N - 2, L = N - 1, NU = 2 + 4 * M;
-  const int e = blockIdx.x * kBlock + threadIdx.x;
-  if (e >= count) return;
-  const uint64_t ev = first + (uint64_t)e;
+  const int e = blockIdx.x * kBlock + threadIdx.x;  // column
+  if (e >= *B.n) return;
+  const uint64_t ev = first + (uint64_t)B.orig[e];
   GradKinF<N> K;
   grad_kin_f32<N>(G.P, G.u + ev * NU, G.order + ev * N, K);
   const uint32_t hel = G.hel[ev];
@@ -507,7 +539,7 @@ __host__ __device__ constexpr int grad_lanes() {
 template <int N>
 __host__ inline int grad_chunk_cap(uint64_t n_events, size_t chunk_bytes) {
   constexpr int L = N - 1;
-  const size_t per_event = (size_t)2 * InRows<L>::rows * sizeof(float) + sizeof(double);
+  const size_t per_event = (size_t)2 * InRows<L>::rows * sizeof(float) + sizeof(double) + sizeof(int);
   const uint64_t bytes = chunk_bytes ? chunk_bytes : ((uint64_t)TESS_GRAD_CHUNK_MB << 20);
   const uint64_t target = std::min<uint64_t>(std::max<uint64_t>(128, (bytes / per_event) / 128 * 128),
                                              (uint64_t)INT32_MAX / 256 * 128);
@@ -519,7 +551,8 @@ template <int N>
 __host__ inline size_t grad_buffer_bytes(int cap) {
   constexpr int L = N - 1;
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
-  return 2 * al((size_t)InRows<L>::rows * cap * sizeof(float)) + al((size_t)cap * sizeof(double));
+  return 2 * al((size_t)InRows<L>::rows * cap * sizeof(float)) + al((size_t)cap * sizeof(double)) +
+         al((size_t)cap * sizeof(int)) + al(sizeof(int));
 }
 
 // One chunk buffer when a single chunk holds every event, else two.
@@ -535,7 +568,7 @@ __host__ inline size_t grad_workspace_bytes(uint64_t n_events, size_t chunk_byte
 // stream, G3 of chunk c (aux stream) runs beside G1/G2 of chunk c+1 (caller's
 // stream): the amplitude stage is held to few warps per SM by its shared
 // tables, and the output stage fills the issue slots it leaves.  Buffer c % 2
-// is rewritten by G2 of chunk c only after G3 of chunk c-2 has read it.
+// is rewritten by chunk c only after G3 of chunk c-2 has read it.
 template <int N>
 cudaError_t launch_grad_n(bool fp64, const GradParams &G, void *ws, cudaStream_t s, const GradStreams &gs) {
   if (fp64) {
@@ -554,30 +587,45 @@ cudaError_t launch_grad_n(bool fp64, const GradParams &G, void *ws, cudaStream_t
     BB[b].in = (float *)base;
     BB[b].gr = (float *)(base + al((size_t)InRows<L>::rows * cap * sizeof(float)));
     BB[b].f = (double *)((char *)BB[b].gr + al((size_t)InRows<L>::rows * cap * sizeof(float)));
+    BB[b].orig = (int *)((char *)BB[b].f + al((size_t)cap * sizeof(double)));
+    BB[b].n = (int *)((char *)BB[b].orig + al((size_t)cap * sizeof(int)));
   }
+  // The number of columns is known on the device alone: the thread-per-event
+  // stages are launched for every event (blocks past the columns end at once),
+  // the amplitude stage with the blocks that are resident at a time, which loop.
   cudaError_t e = cudaSuccess;
+  constexpr size_t amp_smem = GradPairSmem<L, NEV, LN>::bytes;
+  auto amp_grid = [&](auto kernel) {
+    int per_sm = 0;
+    if ((e = allow_max_smem((const void *)kernel)) == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, LN * NEV, amp_smem);
+    const int tiles = (int)((std::min<uint64_t>((uint64_t)cap, G.n_events) + NEV - 1) / NEV);
+    return (unsigned)std::max(1, std::min(tiles, G.sm_count * std::max(per_sm, 1)));
+  };
   if (!G.dw_du && !G.dw_dk && !G.dw_dlnmu) {  // weights alone: one buffer, two kernels per chunk
     if (!G.w) return cudaSuccess;
+    unsigned grid = 0;
     if constexpr (N > 8) {
-      if ((e = allow_max_smem((const void *)grad_amp_kernel<N, NEV, LN, true>)) != cudaSuccess) return e;
+      grid = amp_grid(grad_amp_kernel<N, NEV, LN, true>);
+      if (e != cudaSuccess) return e;
     }
     const GradChunk &B = BB[0];
     for (uint64_t off = 0; off < G.n_events; off += (uint64_t)cap) {
       const int count = (int)std::min<uint64_t>((uint64_t)cap, G.n_events - off);
       const unsigned tb = (unsigned)((count + kBlock - 1) / kBlock);
+      if ((e = cudaMemsetAsync(B.n, 0, sizeof(int), s)) != cudaSuccess) return e;
       grad_in_kernel<N, true><<<tb, kBlock, 0, s>>>(G, off, count, B);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       if constexpr (N <= 8)
-        grad_weight_kernel<N><<<tb, kBlock, 0, s>>>(count, B, G.w + off);
+        grad_weight_kernel<N><<<tb, kBlock, 0, s>>>(B, G.w + off);
       else
-        grad_amp_kernel<N, NEV, LN, true>
-            <<<(unsigned)((count + NEV - 1) / NEV), LN * NEV, GradPairSmem<L, NEV, LN>::bytes, s>>>(count, B,
-                                                                                                   G.w + off);
+        grad_amp_kernel<N, NEV, LN, true><<<grid, LN * NEV, amp_smem, s>>>(B, G.w + off);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
   }
-  if ((e = allow_max_smem((const void *)grad_amp_kernel<N, NEV, LN, false>)) != cudaSuccess) return e;
+  const unsigned ampg = amp_grid(grad_amp_kernel<N, NEV, LN, false>);
+  if (e != cudaSuccess) return e;
   const bool ovl = nbuf == 2 && gs.aux != nullptr;
   if (ovl && ((e = cudaEventRecord(gs.fork, s)) != cudaSuccess || (e = cudaStreamWaitEvent(gs.aux, gs.fork, 0)) != cudaSuccess))
     return e;
@@ -587,20 +635,21 @@ cudaError_t launch_grad_n(bool fp64, const GradParams &G, void *ws, cudaStream_t
     const GradChunk &B = BB[b];
     const int count = (int)std::min<uint64_t>((uint64_t)cap, G.n_events - off);
     const unsigned tb = (unsigned)((count + kBlock - 1) / kBlock);
-    grad_in_kernel<N, false><<<tb, kBlock, 0, s>>>(G, off, count, B);
+    // the buffer's column list is still read by G3 of chunk c-2
     if (ovl && c >= 2 && (e = cudaStreamWaitEvent(s, gs.g3done[b], 0)) != cudaSuccess) return e;
-    grad_amp_kernel<N, NEV, LN, false>
-        <<<(unsigned)((count + NEV - 1) / NEV), LN * NEV, GradPairSmem<L, NEV, LN>::bytes, s>>>(count, B, nullptr);
+    if ((e = cudaMemsetAsync(B.n, 0, sizeof(int), s)) != cudaSuccess) return e;
+    grad_in_kernel<N, false><<<tb, kBlock, 0, s>>>(G, off, count, B);
+    grad_amp_kernel<N, NEV, LN, false><<<ampg, LN * NEV, amp_smem, s>>>(B, nullptr);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    cudaStream_t so = s;
     if (ovl) {
-      if ((e = cudaEventRecord(gs.g2done[b], s)) != cudaSuccess || (e = cudaStreamWaitEvent(gs.aux, gs.g2done[b], 0)) != cudaSuccess)
+      so = gs.aux;
+      if ((e = cudaEventRecord(gs.g2done[b], s)) != cudaSuccess || (e = cudaStreamWaitEvent(so, gs.g2done[b], 0)) != cudaSuccess)
         return e;
-      grad_out_kernel<N><<<tb, kBlock, 0, gs.aux>>>(G, off, count, B);
-      if ((e = cudaGetLastError()) != cudaSuccess || (e = cudaEventRecord(gs.g3done[b], gs.aux)) != cudaSuccess) return e;
-    } else {
-      grad_out_kernel<N><<<tb, kBlock, 0, s>>>(G, off, count, B);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
+    grad_out_kernel<N><<<tb, kBlock, 0, so>>>(G, off, B);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (ovl && (e = cudaEventRecord(gs.g3done[b], so)) != cudaSuccess) return e;
   }
   if (ovl && ((e = cudaEventRecord(gs.join, gs.aux)) != cudaSuccess || (e = cudaStreamWaitEvent(s, gs.join, 0)) != cudaSuccess))
     return e;

@@ -1,0 +1,96 @@
+"""tess_gradients asked for weights alone (no reverse sweep) against the full
+call, and what both write for events that fail the cuts (only the others reach
+the amplitude stage): sizes around the block of 128 and the tile of 32 events,
+none, a tenth and a third of them passing, several chunks."""
+import numpy as np
+import pytest
+import torch
+
+import paper_1002_3446_gb300 as tess
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = tess.tess_init(0)
+    yield c
+    tess.tess_destroy(c)
+
+
+def _draws(ctx, n, N):
+    u, hel, order = tess.tess_draws(ctx, n, 3, 100, N)
+    return u, hel, order
+
+
+def _call(ctx, proc, u, hel, order, names):
+    """tess_gradients into arrays that hold NaN before the call."""
+    E, n = u.shape[0], proc.n_gluons
+    shape = dict(w=(E,), dw_du=(E, u.shape[1]), dw_dk=(E, n, 4), dw_dlnmu=(E,))
+    out = {k: torch.full(shape[k], float("nan"), dtype=torch.float64, device="cuda") for k in names}
+    need = tess.tess_gradients_workspace_size(ctx, proc, E)
+    ws = torch.full(((need + 7) // 8,), float("nan"), dtype=torch.float64, device="cuda") if need else None
+    p = lambda k: tess._ptr(out.get(k))
+    import ctypes
+    tess._check(tess._load().tess_gradients(ctx, ctypes.byref(proc), E, tess._ptr(u), tess._ptr(hel), tess._ptr(order),
+                                            None, p("w"), p("dw_du"), p("dw_dk"), p("dw_dlnmu"), tess._ptr(ws), need,
+                                            tess._stream(None)))
+    torch.cuda.synchronize()
+    return {k: v.cpu().numpy() for k, v in out.items()}
+
+
+ALL = ("w", "dw_du", "dw_dk", "dw_dlnmu")
+
+
+@pytest.mark.parametrize("n", [4, 6, 8, 9, 12])
+@pytest.mark.parametrize("precision", [tess.TESS_FP64, tess.TESS_FP32_DS])
+@pytest.mark.parametrize("N", [1, 31, 33, 127, 129, 1000])
+def test_weights_alone_and_failing_events(ctx, n, precision, N):
+    proc = tess.process(n, precision=precision)
+    u, hel, order = _draws(ctx, n, N)
+    full = _call(ctx, proc, u, hel, order, ALL)
+    alone = _call(ctx, proc, u, hel, order, ("w",))
+    # the same amplitude from a recursion summed in another order (FP32 from n = 4 to
+    # 8, see the parity tests' 99th percentile; the same kernel otherwise)
+    big = np.abs(full["w"]) > 1e-12 * max(np.abs(full["w"]).max(), 1e-300)
+    rel = np.abs(alone["w"][big] / full["w"][big] - 1)
+    assert np.array_equal(alone["w"] == 0, full["w"] == 0)
+    assert rel.size == 0 or (np.median(rel) < 1e-4 and np.linalg.norm(alone["w"] - full["w"]) <=
+                             1e-3 * np.linalg.norm(full["w"]))
+    fail = full["w"] == 0
+    for k in ALL[1:]:
+        assert np.all(np.isfinite(full[k])) and np.all(full[k][fail] == 0)
+
+
+@pytest.mark.parametrize("pt_min,expect", [(1.0, "third"), (3000.0, "none")])
+def test_a_third_or_no_events_pass(ctx, pt_min, expect):
+    n, N = 6, 300
+    proc = tess.process(n, precision=tess.TESS_FP32_DS, pt_min=pt_min, eta_max=50.0, dr_min=0.0)
+    u, hel, order = _draws(ctx, n, N)
+    if expect == "none":
+        proc.sqrt_s = 4 * 3000.0 * 1.0001  # the draws' x reach no such momenta
+    got = _call(ctx, proc, u, hel, order, ALL)
+    assert np.all(np.isfinite(got["w"]))
+    if expect == "none":
+        for k in ALL:
+            assert np.all(got[k] == 0)
+    else:
+        assert np.mean(got["w"] != 0) > 0.2
+
+
+def test_chunks_of_the_column_list(ctx):
+    """Several chunks in two buffers on two streams: the same bits as one chunk."""
+    n, N = 7, 20_001
+    proc = tess.process(n, precision=tess.TESS_FP32_DS)
+    u, hel, order = _draws(ctx, n, N)
+    one = _call(ctx, proc, u, hel, order, ALL)
+    w1 = _call(ctx, proc, u, hel, order, ("w",))
+    try:
+        tess.tess_set_chunk_bytes(ctx, 1 << 20)
+        many = _call(ctx, proc, u, hel, order, ALL)
+        w2 = _call(ctx, proc, u, hel, order, ("w",))
+    finally:
+        tess.tess_set_chunk_bytes(ctx, 0)
+    for k in ALL:
+        assert np.array_equal(one[k], many[k])
+    assert np.array_equal(w1["w"], w2["w"])
