@@ -367,9 +367,11 @@ int tess_autotune_outputs(tess_ctx *ctx, const tess_process *proc, uint64_t prob
                           int *form_out);
 
 /* Sets the variant for (precision, polarisation kind, n) of proc without
- * timing (Sec. 2 running configuration, chosen by the caller): form one of TESS_K2_* (-1: built-in default; a form not built for
+ * timing (Sec. 2 running configuration, chosen by the caller): form one of TESS_K2_* (-1: built-in default, which
+ * follows n, the polarisation kind and the kinematics form; a form not built for
  * (precision, n) or, for the real-current forms, for helicity vectors falls
- * back to the default), schedule one of TESS_SCHED_* (-1: default, serial).
+ * back to the default), schedule one of TESS_SCHED_* (-1: serial, with the histogram
+ * deferred where the default variant is one that gains by it).
  * Takes effect for later calls; TESS_E_INVALID for values out of range.  A
  * workspace sized by tess_workspace_size covers every choice. */
 int tess_select_variant(tess_ctx *ctx, const tess_process *proc, int form, int schedule);

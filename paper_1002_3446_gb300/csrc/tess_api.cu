@@ -563,7 +563,11 @@ int tess_kernel_launches(const tess_ctx *ctx, const tess_process *proc, uint64_t
   if (uses_pipeline(proc)) {
     tess::PipePlan pl;
     if ((rc = pipeline_plan(ctx, proc, n_events, &pl))) return rc;
-    *launches = 2 * pl.chunks + 1;  // (kinematics, amplitude) per chunk + finalize
+    // per chunk the kinematics (with cut-first its scan and index) and the amplitude kernel, or the fused one, and a
+    // deferred histogram's; per call the fold and the grid mode's tables
+    const bool cut_first = (proc->flags & TESS_FLAG_CUT_FIRST) != 0;
+    const int per_chunk = pl.form == tess::K2_FUSED ? 1 : 2 + (cut_first ? 2 : 0) + (pl.defer_hist ? 1 : 0);
+    *launches = per_chunk * pl.chunks + 1 + ((proc->flags & TESS_FLAG_PDF_GRID) ? 1 : 0);
   } else {
     *launches = 2;  // fused event kernel + finalize
   }

@@ -242,9 +242,43 @@ constexpr bool k2_valid(int f, unsigned caps) {
   }
 }
 
+// The variant of a call whose context has none selected (or one that is not
+// built for it), by n, polarisation kind and kinematics.  Times of a whole call in
+// us, 2^20 events unless noted, against the runner-up and, from n = 8, the row
+// form (ROWS32):
+//   helicity vectors   n = 4  FUSED 111 (REG_TMA_HI 115); 1,000 events 16.5 (20.8,
+//                      it saves a launch), n = 5 160 (REG_HI_PF 157; 17.8, 21.5),
+//                      n = 6 225 (REG_HI 225; 19.8, 25.0)
+//                      n = 7  REG 330 (REG_TMA 332), n = 8 REG 514 (WAVE2U 687, ROWS32 772)
+//                      n = 9  WAVE2U 883 (WAVE2PU 1059, ROWS32 1519), n = 10 1191
+//                      (1450, 1915), n = 11 2282 (2462, 3900)
+//                      n = 12 WAVE2PU 3445 (LANES8 3981, ROWS32 8996)
+//   real vectors       n <= 7 REAL_HI 119 / 156 / 201 / 261 (REG 125 / 177 / 258 / 351),
+//                      n = 8, 9 REAL 341 / 447 (ROWS_REAL 364 / 496, ROWS32 792 / 1546)
+//                      n >= 10 ROWS_REAL 771 / 1024 / 1548 (ROWS32 1950 / 3914 / 9036)
+// An event's result must not depend on the size of the call it is part of, so the
+// choice follows the number of events only between FUSED and REG_HI, which give the
+// same bits: without a histogram FUSED loses from 2^22 events (n = 4 / 5 / 6: 380 /
+// 578 / 841 us, REG_HI 372 / 534 / 791), with one it does not (391 / 586 / 855, REG_HI
+// 437 / 596 / 863).  (At 1,000 events and n = 8 / 10 / 12 LANES16 would take 30 / 36 / 40
+// us, the choice below 31 / 42 / 59, ROWS32 35 / 56 / 103.)
 template <int N, typename R>
-constexpr int k2_default() {
-  return sizeof(R) == 8 ? K2_LOOP : (N <= 7 ? K2_REG : K2_ROWS32);
+int k2_default(unsigned caps, int sched, uint64_t n_events, int hist_bins) {
+  if constexpr (sizeof(R) == 8) return K2_LOOP;
+  const bool real_eps = (caps & CAP_REAL_EPS) != 0;
+  if (real_eps) return N <= 7 ? K2_REAL_HI : (N <= 9 ? K2_REAL : K2_ROWS_REAL);
+  if (N <= 6) {
+    const bool fused = k2_valid<N, R>(K2_FUSED, caps) && sched <= SCHED_SERIAL;
+    return fused && (hist_bins > 0 || n_events <= (1u << 21)) ? K2_FUSED : K2_REG_HI;
+  }
+  return N <= 8 ? K2_REG : (N <= 11 ? K2_WAVE2U : K2_WAVE2PU);
+}
+
+// The schedule that goes with it: the forms with long unrolled bodies leave the
+// histogram to its own kernel (see SCHED_SERIAL_HIST; 2^20 events with 40 bins at
+// n = 9 / 10 / 11 / 12: 906 / 1215 / 2332 / 3479 us against 1122 / 1630 / - / 3552).
+inline int k2_default_sched(int form) {
+  return form == K2_WAVE2U || form == K2_WAVE2PU || form == K2_ROWS_REAL ? SCHED_SERIAL_HIST : SCHED_SERIAL;
 }
 
 template <int N, typename R, int F>
@@ -428,14 +462,17 @@ template <int N, typename R>
 int plan_pipeline_t(int sm_count, uint64_t n_events, int hist_bins, int form, int sched, unsigned caps,
                     PipePlan *pl) {
   constexpr int L = N - 1;
-  if (!k2_valid<N, R>(form, caps)) form = k2_default<N, R>();
+  if (!k2_valid<N, R>(form, caps)) {
+    form = k2_default<N, R>(caps, sched, n_events, hist_bins);
+    if (sched < 0) sched = k2_default_sched(form);
+  }
   if (form == K2_FUSED) {
     // its register split (setmaxnreg) assumes the launch's 128 registers a
     // thread; any other compiled count and the form is not offered
     cudaFuncAttributes fa;
     const cudaError_t e = with_form<N, R>(form, [&](auto K) { return cudaFuncGetAttributes(&fa, decltype(K)::fn()); });
     if (e != cudaSuccess) return (int)e;
-    if (fa.numRegs != kFusedLaunchRegs) form = k2_default<N, R>();
+    if (fa.numRegs != kFusedLaunchRegs) form = K2_REG_HI;
   }
   pl->form = form;
   const bool fused = form == K2_FUSED;

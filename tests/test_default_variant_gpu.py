@@ -1,0 +1,49 @@
+"""The built-in amplitude variant and schedule per n, polarisation kind,
+kinematics form, events and histogram, and that an explicit schedule gets a
+variant that can run it."""
+import pytest
+
+import paper_1002_3446_gb300 as tess
+
+pytestmark = pytest.mark.gpu
+
+S, R = tess.TESS_HEL_SAMPLE, tess.TESS_POL_RANDOM
+DS, F32, F64 = tess.TESS_FP32_DS, tess.TESS_FP32_CURRENTS, tess.TESS_FP64
+
+
+def _plan(ctx, n, prec, mode, N, bins=0, flags=0):
+    return tess.tess_plan_info(ctx, tess.process(n, precision=prec, helicity_mode=mode, hist_bins=bins, flags=flags), N)
+
+
+@pytest.mark.parametrize("n,prec,mode,N,bins,flags,variant,schedule", [
+    (4, DS, S, 1000, 0, 0, tess.TESS_K2_FUSED, 0), (6, DS, S, 1 << 21, 0, 0, tess.TESS_K2_FUSED, 0),
+    (6, DS, S, (1 << 21) + 1, 0, 0, tess.TESS_K2_REG_HI, 0), (6, DS, S, 1 << 24, 40, 0, tess.TESS_K2_FUSED, 0),
+    (5, F32, S, 1000, 0, 0, tess.TESS_K2_REG_HI, 0), (6, DS, S, 1000, 0, tess.TESS_FLAG_CUT_FIRST, tess.TESS_K2_REG_HI, 0),
+    (6, DS, R, 1000, 0, 0, tess.TESS_K2_REAL_HI, 0), (7, DS, S, 1000, 40, 0, tess.TESS_K2_REG, 0),
+    (7, F32, R, 1000, 0, 0, tess.TESS_K2_REAL_HI, 0), (8, DS, S, 1000, 40, 0, tess.TESS_K2_REG, 0),
+    (8, F32, R, 1000, 0, 0, tess.TESS_K2_REAL, 0), (9, DS, R, 1000, 40, 0, tess.TESS_K2_REAL, 0),
+    (9, DS, S, 1000, 0, 0, tess.TESS_K2_WAVE2U, 0), (10, DS, S, 1000, 40, 0, tess.TESS_K2_WAVE2U, 4),
+    (11, F32, S, 1000, 40, tess.TESS_FLAG_CUT_FIRST, tess.TESS_K2_WAVE2U, 0),
+    (12, DS, S, 1000, 40, 0, tess.TESS_K2_WAVE2PU, 4), (10, DS, R, 1000, 40, 0, tess.TESS_K2_ROWS_REAL, 4),
+    (12, DS, R, 1000, 0, 0, tess.TESS_K2_ROWS_REAL, 0), (4, F64, S, 1000, 40, 0, tess.TESS_K2_LOOP, 0),
+    (12, F64, R, 1000, 0, 0, tess.TESS_K2_LOOP, 0)])
+def test_default(n, prec, mode, N, bins, flags, variant, schedule):
+    ctx = tess.tess_init(0)
+    try:
+        info = _plan(ctx, n, prec, mode, N, bins, flags)
+        assert (info["variant"], info["schedule"]) == (variant, schedule)
+    finally:
+        tess.tess_destroy(ctx)
+
+
+def test_overlapped_and_tiled_schedules_get_two_kernels():
+    ctx = tess.tess_init(0)
+    try:
+        p = tess.process(6, precision=DS)
+        tess.tess_set_chunk_bytes(ctx, 1 << 20)
+        for s in range(1, 4):
+            tess.tess_select_variant(ctx, p, -1, s)
+            info = tess.tess_plan_info(ctx, p, 100_000)
+            assert info["variant"] == tess.TESS_K2_REG_HI and info["schedule"] == s
+    finally:
+        tess.tess_destroy(ctx)
