@@ -95,6 +95,39 @@ __device__ __forceinline__ float unit_f32(uint32_t a, uint32_t b) {
   return fminf(u, 0x1.fffffep-1f);
 }
 
+// Conversions between binary32 and binary64 on the integer pipe (the native
+// ones share the 1/64-rate FP64 pipe).
+// Rare paths of the conversions below, kept out of line: the compiler cannot
+// turn a call into a predicated select, so the FP64 instructions in them are
+// issued only when taken.
+static __device__ __noinline__ float f32_of_f64_native(double x) { return (float)x; }
+static __device__ __noinline__ double f64_of_f32_native(float x, int k) { return ldexp((double)x, k); }
+
+// binary64 -> binary32, round to nearest even, in integer operations; exact
+// for results in the normal binary32 range (the native conversion otherwise).
+__device__ __forceinline__ float f32_of_f64(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7ffu) - 896;  // rebiased for binary32
+  if (e < 1 || e > 254) return f32_of_f64_native(x);
+  const uint32_t m = ((hi & 0xfffffu) << 3) | (lo >> 29);  // leading 23 mantissa bits
+  const uint32_t rest = lo & 0x1fffffffu;                   // the 29 dropped bits
+  const uint32_t up = (rest > 0x10000000u) | ((rest == 0x10000000u) & (m & 1u));
+  // a carry out of the mantissa steps the exponent, as the rounding requires
+  return __uint_as_float((hi & 0x80000000u) | (((uint32_t)e << 23) + m + up));
+}
+
+// x 2^k as binary64 for binary32 x, in integer operations; exact when x is
+// zero or normal and x 2^k is a normal double (ldexp otherwise).
+__device__ __forceinline__ double f64_of_f32_scaled(float x, int k) {
+  const uint32_t b = __float_as_uint(x);
+  const uint32_t s = b & 0x80000000u;
+  if ((b & 0x7fffffffu) == 0u) return __hiloint2double((int)s, 0);
+  const int e = (int)((b >> 23) & 0xffu);
+  const int E = e + 896 + k;
+  if (e == 0 || e == 255 || E < 1 || E > 2046) return f64_of_f32_native(x, k);
+  return __hiloint2double((int)(s | ((uint32_t)E << 20) | ((b & 0x7fffffu) >> 3)), (int)(b << 29));
+}
+
 // Single uniform j of an event (used for scattered draws).
 __device__ __forceinline__ double uniform_at(uint64_t seed, uint64_t ev, uint32_t j) {
   const double2 p = uniform_pair(seed, ev, j >> 1);

@@ -588,7 +588,7 @@ cudaError_t run_pipeline_t(const EventParams &P, const PipePlan &pl, char *ws, c
   EventParams PG = P;
   if (P.pdf_grid) {  // tables for this call's process
     float *g = (float *)(ws + pl.off_tables);
-    grid_fill_kernel<256><<<(kPdfNodes + kAsNodes + 255) / 256, 256, 0, s>>>(P, g);
+    grid_fill_kernel<32><<<(kPdfNodes + kAsNodes + 31) / 32, 32, 0, s>>>(P, g);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     PG.grid_pdf = g;
     PG.grid_as = g + kPdfNodes;

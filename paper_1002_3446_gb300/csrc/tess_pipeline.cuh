@@ -158,16 +158,19 @@ __device__ __forceinline__ float alphas_f32(const EventParams &P, float ht) {
 
 // Grid mode (Sec. 3's tabulated PDF and alpha_s): the tables, built once per
 // call from the functions in FP64 and rounded to FP32 ...
+// (x^-0.2 from ln x, in which the nodes are uniform; small blocks, since each
+// thread is one serial chain of FP64 work).
 template <int NT>
 __global__ void __launch_bounds__(NT) grid_fill_kernel(EventParams P, float *g) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < kPdfNodes) {
-    const double x = exp((double)i / (double)kPdfSegments * P.lnxmin);
-    g[i] = (float)(1.7 * pow(x, -0.2) * pow(1.0 - x, 5.0));
+    const double lnx = (double)i / (double)kPdfSegments * P.lnxmin;
+    const double t = 1.0 - exp(lnx), t2 = t * t;
+    g[i] = (float)(1.7 * exp(-0.2 * lnx) * (t2 * t2 * t));
   } else if (i < kPdfNodes + kAsNodes) {
     const int j = i - kPdfNodes;
-    const double mu = exp(0.5 * (P.as_vlo + (P.as_vhi - P.as_vlo) * j / (double)kAsSegments));
-    g[i] = (float)(P.alphas_mz / (1.0 + P.alphas_mz * P.b0 * (log(mu * mu) - P.ln_mz2)));
+    const double lnmu2 = P.as_vlo + (P.as_vhi - P.as_vlo) * j / (double)kAsSegments;
+    g[i] = (float)(P.alphas_mz / (1.0 + P.alphas_mz * P.b0 * (lnmu2 - P.ln_mz2)));
   }
 }
 
@@ -295,24 +298,34 @@ __device__ __forceinline__ void kin_fp64(const ChunkParams &C, const ChunkBuf<do
 // Polarisation basis of an outgoing massless momentum (E, px, py, pz) in FP64
 // (the Gram products): e1 = theta-hat = (ct cf, ct sf, -st), e2 = phi-hat =
 // (-sf, cf, 0), with ct = pz/E, st = pT/E, cf = px/pT, sf = py/pT (E = |p|
-// for a massless momentum).  Returned rounded to FP32.
+// for a massless momentum).  Returned rounded to FP32, so the reciprocals take
+// one FP64 Newton step from their FP32 estimates (2^-45; 15 FP64 operations for
+// 30 with full-length ones and native conversions).
 __device__ __forceinline__ void pol_basis_f32(double E, double px, double py, double pz, float (&e1)[3],
                                               float (&e2)[2]) {
   const double pt2 = px * px + py * py;
   double cf = 1.0, sf = 0.0, pt = 0.0;
   if (pt2 > 0.0) {
-    const double inv_pt = rsqrt(pt2);
-    pt = pt2 * inv_pt;
-    cf = px * inv_pt;
-    sf = py * inv_pt;
+    const float p2 = f32_of_f64(pt2);
+    double ipt;
+    if (p2 > 0x1p-100f) {
+      const double y = f64_of_f32_scaled(rsqrtf(p2), 0);
+      ipt = fma(0.5 * y, fma(-(pt2 * y), y, 1.0), y);
+    } else {
+      ipt = rsqrt(pt2);
+    }
+    pt = pt2 * ipt;
+    cf = px * ipt;
+    sf = py * ipt;
   }
-  const double inv_e = 1.0 / E;
+  const double r = f64_of_f32_scaled(1.f / f32_of_f64(E), 0);
+  const double inv_e = fma(r, fma(-E, r, 1.0), r);
   const double ct = pz * inv_e, st = pt * inv_e;
-  e1[0] = (float)(ct * cf);
-  e1[1] = (float)(ct * sf);
-  e1[2] = (float)(-st);
-  e2[0] = (float)(-sf);
-  e2[1] = (float)cf;
+  e1[0] = f32_of_f64(ct * cf);
+  e1[1] = f32_of_f64(ct * sf);
+  e1[2] = f32_of_f64(-st);
+  e2[0] = f32_of_f64(-sf);
+  e2[1] = f32_of_f64(cf);
 }
 
 // Writes the amplitude inputs of one event -- per colour position a: the leg
@@ -462,11 +475,12 @@ __device__ __forceinline__ void kin_fp32(const ChunkParams &C, const ChunkBuf<fl
   const float ux1 = unit_f32(w0.x, w0.y), ux2 = unit_f32(w0.z, w0.w);
   const float x1 = expf(ux1 * lnxmin);
   const float x2 = expf(ux2 * lnxmin);
-  const double shat = (double)x1 * (double)x2 * P.S;
+  const double shat = f64_of_f32_scaled(x1, 0) * f64_of_f32_scaled(x2, 0) * P.S;
   const double rs = sqrt(shat);
 
-  // Rambo seeds in FP32, boost + rescale in FP64
-  float qf[M][4];
+  // Rambo seeds in FP32, boost + rescale in FP64 (whose pipe bounds the kernel:
+  // conversions run on the integer pipe)
+  double qd[M][4];
   double Q0 = 0.0, Q1 = 0.0, Q2 = 0.0, Q3 = 0.0;
 #pragma unroll
   for (int i = 0; i < M; ++i) {
@@ -477,14 +491,14 @@ __device__ __forceinline__ void kin_fp32(const ChunkParams &C, const ChunkBuf<fl
     float sn, cs;
     sincospif(2.f * unit_f32(wa.z, wa.w), &sn, &cs);
     const float q0 = -logf(unit_f32(wb.x, wb.y) * unit_f32(wb.z, wb.w));
-    qf[i][0] = q0;
-    qf[i][1] = q0 * sn0 * cs;
-    qf[i][2] = q0 * sn0 * sn;
-    qf[i][3] = q0 * c;
-    Q0 += (double)qf[i][0];
-    Q1 += (double)qf[i][1];
-    Q2 += (double)qf[i][2];
-    Q3 += (double)qf[i][3];
+    qd[i][0] = f64_of_f32_scaled(q0, 0);
+    qd[i][1] = f64_of_f32_scaled(q0 * sn0 * cs, 0);
+    qd[i][2] = f64_of_f32_scaled(q0 * sn0 * sn, 0);
+    qd[i][3] = f64_of_f32_scaled(q0 * c, 0);
+    Q0 += qd[i][0];
+    Q1 += qd[i][1];
+    Q2 += qd[i][2];
+    Q3 += qd[i][3];
   }
   const double invM = rsqrt(Q0 * Q0 - Q1 * Q1 - Q2 * Q2 - Q3 * Q3);
   const double bx = -Q1 * invM, by = -Q2 * invM, bz = -Q3 * invM;
@@ -494,7 +508,7 @@ __device__ __forceinline__ void kin_fp32(const ChunkParams &C, const ChunkBuf<fl
   double pk[M][4];
 #pragma unroll
   for (int i = 0; i < M; ++i) {
-    const double q0 = qf[i][0], q1 = qf[i][1], q2 = qf[i][2], q3 = qf[i][3];
+    const double q0 = qd[i][0], q1 = qd[i][1], q2 = qd[i][2], q3 = qd[i][3];
     const double bq = bx * q1 + by * q2 + bz * q3;
     pk[i][0] = xs * (gam * q0 + bq);
     const double f = aa * bq + q0;
@@ -505,14 +519,15 @@ __device__ __forceinline__ void kin_fp32(const ChunkParams &C, const ChunkBuf<fl
 
   // cuts and observables in FP32
   const float y = __fmul_rn(0.5f, logf(__fdiv_rn(x1, x2)));
-  float eta[M], phi[M];
+  float eta[M], phi[M], pkf[M][4];
   int pass = 1;
   float sum = 0.f, lead = 0.f;
 #pragma unroll
   for (int i = 0; i < M; ++i) {
-    const float pkf[4] = {(float)pk[i][0], (float)pk[i][1], (float)pk[i][2], (float)pk[i][3]};
-    cut_observe(P, pkf, y, eta[i], pass, sum, lead);
-    phi[i] = atan2f(pkf[2], pkf[1]);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) pkf[i][m] = f32_of_f64(pk[i][m]);
+    cut_observe(P, pkf[i], y, eta[i], pass, sum, lead);
+    phi[i] = atan2f(pkf[i][2], pkf[i][1]);
   }
   const float dr2min = pair_cuts<M>(P, eta, phi, pass);
   const double ht = (double)sum, ptlead = (double)lead, rmin = (double)sqrtf(dr2min);
@@ -530,33 +545,30 @@ __device__ __forceinline__ void kin_fp32(const ChunkParams &C, const ChunkBuf<fl
   double wf = 0.0;
   if (pass) {
     const float as = P.pdf_grid ? grid_alphas(P, sum) : alphas_f32(P, sum);
-    const double g2 = 4.0 * 3.14159265358979323846 * (double)as;
-    double gp = 1.0;
-#pragma unroll
-    for (int i = 0; i < N - 2; ++i) gp *= g2;
-    double sp = 1.0;
-#pragma unroll
-    for (int i = 0; i < M - 2; ++i) sp *= shat;
+    const double g2 = 4.0 * 3.14159265358979323846 * f64_of_f32_scaled(as, 0);
     const float f1 = P.pdf_grid ? grid_pdf(P, ux1) : 1.7f * powf(x1, -0.2f) * powf(1.f - x1, 5.f);
     const float f2 = P.pdf_grid ? grid_pdf(P, ux2) : 1.7f * powf(x2, -0.2f) * powf(1.f - x2, 5.f);
-    const double lum = P.lnxmin * P.lnxmin * (double)f1 * (double)f2;
-    wf = P.wconst * lum / (2.0 * shat) * (P.phiconst * sp) * gp;
-  }
-  const double inv_rs = pow2_unit_inv(rs);
-  double ef = P.efac;
-  const double u2 = inv_rs * inv_rs;
+    wf = P.wk * (f64_of_f32_scaled(f1, 0) * f64_of_f32_scaled(f2, 0));  // wk = wconst (ln x_min)^2 phiconst / 2
 #pragma unroll
-  for (int i = 0; i < N - 4; ++i) ef *= u2;
-  B.efac[ec] = ef;
+    for (int i = 0; i < N - 2; ++i) wf *= g2;
+    if constexpr (M >= 3) {
+#pragma unroll
+      for (int i = 0; i < M - 3; ++i) wf *= shat;
+    } else {
+      wf /= shat;
+    }
+  }
+  const int ex = exponent_of(rs);  // momentum unit 2^-ex
+  B.efac[ec] = scale_pow2(P.efac, -2 * ex * (N - 4));
   B.wfac[ec] = wf;
   B.pass[ec] = (uint8_t)pass;
-  if (B.hval) B.hval[ec] = P.hist_obs == 0 ? ptlead : (P.hist_obs == 1 ? ht : rmin);
+  if (B.hval && P.hist_bins > 0) B.hval[ec] = P.hist_obs == 0 ? ptlead : (P.hist_obs == 1 ? ht : rmin);
 
   // per-leg FP32 data: momentum in units of the power-of-two scale, and the
   // polarisation basis (e1 spatial, e2 transverse); beam-axis legs are exact
   float lk[N][4], le1[N][3], le2[N][2];
-  const float sc = (float)inv_rs;
-  const float hs = (float)(0.5 * rs) * sc;
+  const float sc = ldexpf(1.f, -ex);
+  const float hs = f32_of_f64(0.5 * rs) * sc;
   lk[0][0] = -hs; lk[0][1] = 0.f; lk[0][2] = 0.f; lk[0][3] = -hs;
   lk[1][0] = -hs; lk[1][1] = 0.f; lk[1][2] = 0.f; lk[1][3] = hs;
   le1[0][0] = 1.f; le1[0][1] = 0.f; le1[0][2] = 0.f; le2[0][0] = 0.f; le2[0][1] = 1.f;   // physical +z
@@ -564,7 +576,7 @@ __device__ __forceinline__ void kin_fp32(const ChunkParams &C, const ChunkBuf<fl
 #pragma unroll
   for (int i = 0; i < M; ++i) {
 #pragma unroll
-    for (int m = 0; m < 4; ++m) lk[2 + i][m] = (float)pk[i][m] * sc;
+    for (int m = 0; m < 4; ++m) lk[2 + i][m] = pkf[i][m] * sc;
     pol_basis_f32(pk[i][0], pk[i][1], pk[i][2], pk[i][3], le1[2 + i], le2[2 + i]);
   }
 
