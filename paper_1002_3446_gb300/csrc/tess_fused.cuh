@@ -125,7 +125,7 @@ __device__ __forceinline__ Cx<float> tile_amplitude(const float *tile, int col) 
 // Block sums of the amplitude warpgroup (col = its thread's column) added to
 // the block's partial row, as epi_flush does for a whole block.
 __device__ __forceinline__ void fused_flush(const EpiSmem<kFusedThreads> &S, int nb2, const Accum<kFusedThreads> &A,
-                                            double *red, double *partials, int hist_bins, int col) {
+                                            double *red, double *partials, const ChunkParams &C, int col) {
   red[0 * kBlock + col] = A.sw;
   red[1 * kBlock + col] = A.sw2;
   red[2 * kBlock + col] = (double)A.npass;
@@ -138,9 +138,10 @@ __device__ __forceinline__ void fused_flush(const EpiSmem<kFusedThreads> &S, int
     }
     nbar_sync<kBarAmpOnly, kBlock>();
   }
-  double *row = partials + (size_t)blockIdx.x * partial_stride(hist_bins);
-  if (col < 4) row[col] += red[col * kBlock];
-  for (int i = col; i < 2 * nb2; i += kBlock) row[kPartialHead + i] += epi_hist_sum(S, nb2, i);
+  double *row = partials + (size_t)blockIdx.x * partial_stride(C.P.hist_bins);
+  if (col < 4) row_add(C, row + col, red[col * kBlock]);
+  if (col == 4) row_add(C, row + 4, 0.0);
+  for (int i = col; i < 2 * nb2; i += kBlock) row_add(C, row + kPartialHead + i, epi_hist_sum(S, nb2, i));
 }
 
 // The chunk's events [C.chunk_first, + C.count) of the call; partial row
@@ -196,7 +197,7 @@ __global__ void __launch_bounds__(kFusedThreads, 2) fused_kernel(const __grid_co
       if (t + 2 * (int)gridDim.x < ntiles) nbar_arrive_stage<kBarEmpty>(b);
       epi_tile<kFusedThreads>(ES, nb2, w, bin);
     }
-    fused_flush(ES, nb2, A, red, partials, C.P.hist_bins, col);
+    fused_flush(ES, nb2, A, red, partials, C, col);
   }
 }
 

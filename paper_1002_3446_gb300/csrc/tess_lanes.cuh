@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(32 * NW) bg_lanes_kernel(ChunkParams C, ChunkB
     if (live && r == 0) finish_event<NB, float>(C, B, e, amp2_of(amp), A, w, bin);
     epi_tile<NB>(ES, nb2, w, bin);
   }
-  epi_flush<NB>(ES, nb2, A, partials, C.P.hist_bins);
+  epi_flush<NB>(ES, nb2, A, partials, C);
 }
 
 }  // namespace tess

@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(2 * NEV) bg_pair_w_kernel(ChunkParams C, Chunk
     epi_tile<NB>(ES, nb2, w, bin);
     __syncthreads();  // the table is refilled by the next tile
   }
-  epi_flush<NB>(ES, nb2, A, partials, C.P.hist_bins);
+  epi_flush<NB>(ES, nb2, A, partials, C);
 }
 
 }  // namespace tess

@@ -583,8 +583,7 @@ template <int N, typename R>
 cudaError_t run_pipeline_t(const EventParams &P, const PipePlan &pl, char *ws, cudaStream_t s,
                            const StageHook *hook, const OverlapRes *ov = nullptr) {
   double *partials = (double *)ws;
-  cudaError_t e = cudaMemsetAsync(partials, 0, (size_t)pl.grid * partial_stride(P.hist_bins) * sizeof(double), s);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
   EventParams PG = P;
   if (P.pdf_grid) {  // tables for this call's process
     float *g = (float *)(ws + pl.off_tables);

@@ -1090,9 +1090,15 @@ __device__ __forceinline__ double epi_hist_sum(const EpiSmem<NB> &S, int nb2, in
   return v;
 }
 
+// Adds v to a block's partial row.  Every block writes its row for every chunk,
+// so the call's first chunk stores: the rows need no clearing before it.
+__device__ __forceinline__ void row_add(const ChunkParams &C, double *q, double v) {
+  *q = C.chunk_first == 0 ? v : *q + v;
+}
+
 template <int NB>
 __device__ __forceinline__ void epi_flush(const EpiSmem<NB> &S, int nb2, Accum<NB> &A, double *partials,
-                                          int hist_bins, int stalled = 0) {
+                                          const ChunkParams &C, int stalled = 0) {
   __shared__ double red[4][NB];
   red[0][threadIdx.x] = A.sw;
   red[1][threadIdx.x] = A.sw2;
@@ -1106,10 +1112,10 @@ __device__ __forceinline__ void epi_flush(const EpiSmem<NB> &S, int nb2, Accum<N
     }
     __syncthreads();
   }
-  double *row = partials + (size_t)blockIdx.x * partial_stride(hist_bins);
-  if (threadIdx.x < 4) row[threadIdx.x] += red[threadIdx.x][0];
-  if (threadIdx.x == 4 && stalled) row[4] += 1.0;
-  for (int i = threadIdx.x; i < 2 * nb2; i += NB) row[kPartialHead + i] += epi_hist_sum(S, nb2, i);
+  double *row = partials + (size_t)blockIdx.x * partial_stride(C.P.hist_bins);
+  if (threadIdx.x < 4) row_add(C, row + threadIdx.x, red[threadIdx.x][0]);
+  if (threadIdx.x == 4) row_add(C, row + 4, stalled ? 1.0 : 0.0);
+  for (int i = threadIdx.x; i < 2 * nb2; i += NB) row_add(C, row + kPartialHead + i, epi_hist_sum(S, nb2, i));
 }
 
 // Deferred histogram (schedule SCHED_SERIAL_HIST): after the amplitude kernel
@@ -1142,7 +1148,7 @@ __global__ void __launch_bounds__(NB) hist_chunk_kernel(ChunkParams C, const dou
   }
   __syncthreads();
   double *row = partials + (size_t)blockIdx.x * partial_stride(C.P.hist_bins);
-  for (int i = threadIdx.x; i < 2 * nb2; i += NB) row[kPartialHead + i] += epi_hist_sum(S, nb2, i);
+  for (int i = threadIdx.x; i < 2 * nb2; i += NB) row_add(C, row + kPartialHead + i, epi_hist_sum(S, nb2, i));
 }
 
 // L2 prefetch, by the whole block, of the amplitude inputs and event factors
@@ -1209,7 +1215,7 @@ __global__ void __launch_bounds__(NB, MINB) bg_reg_kernel(ChunkParams C, ChunkBu
     }
     epi_tile<NB>(S, nb2, w, bin);
   }
-  epi_flush<NB>(S, nb2, A, partials, C.P.hist_bins);
+  epi_flush<NB>(S, nb2, A, partials, C);
 }
 
 // K2, real-current register form (FP32, random real polarisations, n <= 9):
@@ -1255,7 +1261,7 @@ __global__ void __launch_bounds__(NB, MINB) bg_real_kernel(ChunkParams C, ChunkB
     }
     epi_tile<NB>(S, nb2, w, bin);
   }
-  epi_flush<NB>(S, nb2, A, partials, C.P.hist_bins);
+  epi_flush<NB>(S, nb2, A, partials, C);
 }
 
 // K2, staged register form (FP32, n <= 8): as bg_reg_kernel, with each
@@ -1401,7 +1407,7 @@ __global__ void __launch_bounds__(NB, MINB)
     __syncwarp();
   }
   const int stalled = __syncthreads_or(dead) ? 1 : 0;
-  epi_flush<NB>(ES, nb2, A, partials, C.P.hist_bins, stalled);
+  epi_flush<NB>(ES, nb2, A, partials, C, stalled);
 }
 
 // K2, loop form (FP64): table in per-thread local memory.
@@ -1435,7 +1441,7 @@ __global__ void __launch_bounds__(NB) bg_loop_kernel(ChunkParams C, ChunkBuf<dou
     }
     epi_tile<NB>(S, nb2, w, bin);
   }
-  epi_flush<NB>(S, nb2, A, partials, C.P.hist_bins);
+  epi_flush<NB>(S, nb2, A, partials, C);
 }
 
 // ---------------------------------------------------------------------------
@@ -1673,7 +1679,7 @@ __global__ void __launch_bounds__(NB) bg_rows_real_kernel(ChunkParams C, ChunkBu
     }
     epi_tile<NB>(S, nb2, w, bin);
   }
-  epi_flush<NB>(S, nb2, A, partials, C.P.hist_bins);
+  epi_flush<NB>(S, nb2, A, partials, C);
 }
 
 template <int L>
@@ -1719,7 +1725,7 @@ __global__ void __launch_bounds__(NB) bg_rows_kernel(ChunkParams C, ChunkBuf<flo
     }
     epi_tile<NB>(S, nb2, w, bin);
   }
-  epi_flush<NB>(S, nb2, A, partials, C.P.hist_bins);
+  epi_flush<NB>(S, nb2, A, partials, C);
 }
 
 }  // namespace tess

@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(NE * G) bg_wavep_kernel(ChunkParams C, ChunkBu
     if (has && g == G - 1) finish_event<NT, float>(C, B, e, amp2_of(amp), A, w, bin);
     epi_tile<NT>(S, nb2, w, bin);
   }
-  epi_flush<NT>(S, nb2, A, partials, C.P.hist_bins);
+  epi_flush<NT>(S, nb2, A, partials, C);
 }
 
 }  // namespace tess
