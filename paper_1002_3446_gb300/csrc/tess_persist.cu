@@ -5,14 +5,23 @@
 
 #include "tess_persist.cuh"
 
+#include <cooperative_groups.h>
+
+namespace cg = cooperative_groups;
+
 namespace tess {
 
-constexpr int kFoldThreads = 64;
+constexpr int kFoldThreads = 128;
+constexpr int kFoldSlices = 8;  // blocks (one cluster) per column
 
-// Block (q, p): column q of process p's tile rows, each thread over the rows
-// t, t + kFoldThreads, ... with compensation, then a fixed-shape compensated
-// tree (deterministic); folded into the caller's accumulators with their own
-// compensation terms.
+// Cluster (q, p): column q of process p's tile rows, block z of the cluster over
+// the rows z kFoldThreads + t, + kFoldSlices kFoldThreads, ... with compensation
+// per thread, a fixed-shape compensated tree per block, and the cluster's first
+// block adds the others' sums, read from their shared memory, in block order
+// (deterministic); folded into the caller's accumulators with their own
+// compensation terms.  A column is a serial chain of FP64 additions (1/64 of the
+// FP32 rate), so it is the longest column's SM that bounds the fold: one block
+// of 64 threads per column took 62 us for the 8,192 tiles of 2^20 events.
 __device__ __forceinline__ void persist_comp_add(double &s, double &c, double x) {
   const double t = s + x;
   if (fabs(s) >= fabs(x))
@@ -22,14 +31,16 @@ __device__ __forceinline__ void persist_comp_add(double &s, double &c, double x)
   s = t;
 }
 
-__global__ void __launch_bounds__(kFoldThreads) persist_fold_kernel(const __grid_constant__ PersistFold F) {
-  const int p = blockIdx.y, q = blockIdx.x, t = threadIdx.x;
+__global__ void __launch_bounds__(kFoldThreads) __cluster_dims__(1, 1, kFoldSlices)
+    persist_fold_kernel(const __grid_constant__ PersistFold F) {
+  const int p = blockIdx.y, q = blockIdx.x, t = threadIdx.x, z = blockIdx.z;
   const int hb = F.hist_bins[p];
   const int nb2 = hb > 0 ? hb + 2 : 0;
-  if (q >= kPartialHead + 2 * nb2) return;  // uniform per block
+  if (q >= kPartialHead + 2 * nb2) return;  // uniform per cluster
   const int stride = partial_stride(hb);
   double s = 0.0, c = 0.0;
-  for (int r = t; r < F.tiles[p]; r += kFoldThreads) persist_comp_add(s, c, F.tile_sums[p][(size_t)r * stride + q]);
+  for (int r = z * kFoldThreads + t; r < F.tiles[p]; r += kFoldSlices * kFoldThreads)
+    persist_comp_add(s, c, F.tile_sums[p][(size_t)r * stride + q]);
   __shared__ double ss[kFoldThreads], cc[kFoldThreads];
   ss[t] = s;
   cc[t] = c;
@@ -43,8 +54,19 @@ __global__ void __launch_bounds__(kFoldThreads) persist_fold_kernel(const __grid
     }
     __syncthreads();
   }
-  if (t != 0) return;
-  const double tot = ss[0] + cc[0];
+  cg::cluster_group cluster = cg::this_cluster();
+  cluster.sync();  // every block's sums are in its shared memory
+  double tot = 0.0;
+  if (z == 0 && t == 0) {
+    double a = ss[0], ac = cc[0];
+    for (int k = 1; k < kFoldSlices; ++k) {
+      persist_comp_add(a, ac, *cluster.map_shared_rank(&ss[0], k));
+      ac += *cluster.map_shared_rank(&cc[0], k);
+    }
+    tot = a + ac;
+  }
+  cluster.sync();  // the other blocks' shared memory stays until it has been read
+  if (z != 0 || t != 0) return;
   double *acc = F.acc[p], *hist = F.hist[p];
   if (q == 0 || q == 1) {
     double hs = acc[q], hc = acc[4 + q];
@@ -100,7 +122,7 @@ static cudaError_t persist_run(const PersistParams &Q, const PersistFold &F, int
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   int cols = 0;
   for (int p = 0; p < Q.nproc; ++p) cols = std::max(cols, partial_stride(F.hist_bins[p]));
-  persist_fold_kernel<<<dim3(cols, Q.nproc), kFoldThreads, 0, s>>>(F);
+  persist_fold_kernel<<<dim3(cols, Q.nproc, kFoldSlices), kFoldThreads, 0, s>>>(F);
   return cudaGetLastError();
 }
 
