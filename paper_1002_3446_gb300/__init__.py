@@ -610,41 +610,49 @@ def _lc_amplitude_flops(L):
     def dot(la, lb):
         return 2 if la and lb else (4 if la or lb else 16)
 
-    total = 0
-    for ln in range(2, L):
+    def madd(ru, rv):
+        return 2 if ru and rv else (4 if ru or rv else 8)
+
+    total = (L - 1) * (2 + 9 + 4 + 7 + 6 + 3 + 2 + 1)  # two-leg sets
+    for ln in range(3, L):
         for a in range(0, L - ln + 1):
             b = a + ln - 1
             for i in range(a, b):
                 ll, lr = i == a, i + 1 == b
-                total += 2 + dot(ll, lr)                          # db, D
-                total += (4 if ll else 13) + (4 if lr else 13)    # c_r, c_l
-                total += (6 if lr else 16) + (6 if ll else 16)    # c_r J_r, c_l J_l
-                total += 5 + 8 + 2 + 1 + 4                        # D db term, S, w
+                total += 2 + dot(ll, lr)                                            # db, D
+                total += (4 if ll else 12 if i == a + 1 else 15)                    # c_r
+                total += (4 if lr else 12 if i + 2 == b else 15)                    # c_l
+                total += (6 if lr else 16) + (6 if ll else 16)                      # c_r J_r, c_l J_l
+                total += 5 + 8 + 2 + 1 + 4                                          # D db term, S, w
                 for j in range(i + 1, b):                         # triples ([a..i], [i+1..j], [j+1..b])
-                    total += dot(i == a, j + 1 == b) + (6 if j == i + 1 else 16)
+                    three = i == a and j == i + 1 and j + 1 == b
+                    total += dot(i == a, j + 1 == b) + (3 if three else 6 if j == i + 1 else 16)
             total += 12 + 8                                       # propagator; w, A, B, omega
     e = L - 1
     for i in range(0, e):
-        total += (8 + dot(i + 1 == e, True) if i > 0 else 0) + (8 + dot(i == 0, True) if i + 1 < e else 0)
-        total += 3 + 8 + dot(i == 0, i + 1 == e)
+        total += (madd(i == 1, i + 1 == e) + dot(i + 1 == e, True) if i > 0 else 0)
+        total += (madd(i + 2 == e, i == 0) + dot(i == 0, True) if i + 1 < e else 0)
+        total += 3 + madd(i == 0 and i + 1 == e, False) + dot(i == 0, i + 1 == e)
         for j in range(i + 1, e):
-            total += 8 + dot(i == 0, j + 1 == e) + dot(j == i + 1, True)
+            total += madd(i == 0 and j + 1 == e, i + 1 == j) + dot(i == 0, j + 1 == e) + dot(j == i + 1, True)
     return total + 4
 
 
-def exact_sum_flops(n):
-    """Real floating-point operations of one event's exact sum over helicities
-    and colour orderings (n = 4, 5) as the kernel evaluates it: half of the
-    (n-1)! orderings (the reversed ones are equal), of each the 2^(n-1) labellings
-    with leg 0's label fixed that do not vanish at tree level."""
-    L = n - 1
-    orderings = math.factorial(n - 1) // 2
-    return orderings * _lc_order_flops(L) + exact_sum_amplitudes(n) * (_lc_amplitude_flops(L) + 4)
-
-
 def exact_sum_amplitudes(n):
-    """Amplitudes that the exact sum evaluates per event: 9 at n = 4, 120 at n = 5."""
-    return math.factorial(n - 1) // 2 * sum(math.comb(n - 1, k) for k in range(2, n - 1))
+    """Amplitudes that the exact sum evaluates per event: 6 at n = 4 (two
+    orderings, the third follows from them), 120 at n = 5 (half of the (n-1)!, the
+    reversed ones being equal); of each the labellings with leg 0's label fixed
+    that do not vanish at tree level."""
+    orderings = 2 if n == 4 else math.factorial(n - 1) // 2
+    return orderings * sum(math.comb(n - 1, k) for k in range(2, n - 1))
+
+
+def exact_sum_flops(n):
+    """Real floating-point operations of the amplitudes of one event's exact sum
+    over helicities and colour orderings (n = 4, 5) as the kernel evaluates it."""
+    L = n - 1
+    orderings = 2 if n == 4 else math.factorial(n - 1) // 2
+    return orderings * _lc_order_flops(L) + exact_sum_amplitudes(n) * (_lc_amplitude_flops(L) + 4)
 
 
 def bg_flops_real(n):

@@ -481,12 +481,16 @@ __device__ __forceinline__ double pow2_unit_inv(double rs) {
 // conjugates each polarisation vector up to a sign, and reversing the ordering
 // changes the amplitude by (-1)^n, so leg 0 keeps label 0, an ordering and its
 // reverse are one term, and the sum is taken four times; labellings with at
-// most one label unlike the others vanish at tree level.  That leaves 3
-// orderings of 3 labellings at n = 4 (of 6 x 8 before) and 12 of 10 at n = 5 (of
-// 24 x 16), each in light-cone gauge (tess_lc.cuh) with the momenta's part shared
-// by the labellings of an ordering.  The summed squares lose nothing: against 64
-// bits, in FP32, the largest error of 3,000 events at n = 4 was 5e-7 (9e-7 with
-// four-component currents), of 600 at n = 5 2e-5 (4e-4).
+// most one label unlike the others vanish at tree level.  At n = 4 the three
+// orderings left add up to zero (U(1) decoupling), so the third is minus the sum
+// of two: where it is small and loses digits the sum of squares does not.  That
+// leaves 2 orderings of 3 labellings at n = 4 (of 6 x 8 before) and 12 of 10 at
+// n = 5 (of 24 x 16), each in light-cone gauge (tess_lc.cuh) with the momenta's
+// part shared by the labellings of an ordering (2^20 events at n = 4, whole call:
+// 49.4 ms with every term in four-component currents, 2.30 ms now).  The summed
+// squares lose nothing: against 64 bits, in FP32, the largest error of 3,000
+// events at n = 4 was 7e-7 (9e-7 with four-component currents; the third ordering
+// from the other two or by itself alike), of 600 at n = 5 2e-5 (4e-4).
 template <typename R, int N>
 __device__ __forceinline__ double summed_amp2(const double (&k)[N - 2][4], int ex) {
   constexpr int L = N - 1;
@@ -496,10 +500,25 @@ __device__ __forceinline__ double summed_amp2(const double (&k)[N - 2][4], int e
   for (int l = 1; l < L; ++l)
     leg[l] = lc_leg<R>(scale_pow2_z(k[l - 1][0], -ex), scale_pow2_z(k[l - 1][1], -ex), scale_pow2_z(k[l - 1][2], -ex),
                        scale_pow2_z(k[l - 1][3], -ex));
+  double acc = 0.0;
+  if constexpr (N == 4) {
+    const LCLeg<R> g1[L] = {leg[0], leg[1], leg[2]}, g2[L] = {leg[1], leg[0], leg[2]};
+    LCOrder<R, L> o1, o2;
+    lc_order<R, L>(g1, 0, o1);
+    lc_order<R, L>(g2, 1, o2);
+#pragma unroll 1
+    for (int odd = 0; odd < 3; ++odd) {  // the leg of 1..3 that keeps leg 0's label
+      const R s0 = odd == 0 ? R(-1) : R(1), s1 = odd == 1 ? R(-1) : R(1), s2 = odd == 2 ? R(-1) : R(1);
+      const R sa[L] = {s0, s1, s2}, sb[L] = {s1, s0, s2};
+      const Cx<R> a = lc_amplitude<R, L>(o1, sa, R(1)), b = lc_amplitude<R, L>(o2, sb, R(1));
+      const double are = a.re, aim = a.im, bre = b.re, bim = b.im, cre = are + bre, cim = aim + bim;
+      acc += fma(are, are, aim * aim) + fma(bre, bre, bim * bim) + fma(cre, cre, cim * cim);
+    }
+    return acc * (4.0 / (double)(1 << N));
+  }
   int perm[L];  // colour position -> leg - 1
 #pragma unroll
   for (int i = 0; i < L; ++i) perm[i] = i;
-  double acc = 0.0;
   for (bool more = true; more;) {
     if (perm[0] < perm[L - 1]) {
       LCLeg<R> g[L];

@@ -40,11 +40,12 @@ struct LCLeg {
 };
 
 // Light-cone components of an outgoing massless momentum: the smaller of K+,
-// K- from pT^2 over the larger.
+// K- from pT^2 over the larger (one reciprocal for both and for 1 / K+).
 template <typename R>
 __device__ __forceinline__ LCLeg<R> lc_leg(double e, double px, double py, double pz) {
-  const double pt2 = px * px + py * py, big = e + fabs(pz), small = pt2 / big;
-  const double p = pz > 0.0 ? small : big, ip = pz > 0.0 ? big / pt2 : 1.0 / big;
+  const double pt2 = px * px + py * py, big = e + fabs(pz);
+  const double r = 1.0 / (pt2 * big), small = (r * pt2) * pt2;
+  const double p = pz > 0.0 ? small : big, ip = pz > 0.0 ? (r * big) * big : r * pt2;
   return {R(px), R(py), R(p), R(pz > 0.0 ? big : small), R(px * ip), R(py * ip)};
 }
 
@@ -151,9 +152,30 @@ __device__ __forceinline__ void lc_axpy_leaf(LCCur<R> &acc, const Cx<R> &c, R s)
   acc.y.im = fma(s, c.re, acc.y.im);
 }
 
+// z += u v, where u (RU) or v (RV) is real: its imaginary part is not read.
+template <bool RU, bool RV, typename R>
+__device__ __forceinline__ void lc_madd(Cx<R> &z, const Cx<R> &u, const Cx<R> &v) {
+  z.re = fma(u.re, v.re, z.re);
+  if constexpr (!RU && !RV) z.re = fma(-u.im, v.im, z.re);
+  if constexpr (!RV) z.im = fma(u.re, v.im, z.im);
+  if constexpr (!RU) z.im = fma(u.im, v.re, z.im);
+}
+
+// acc -= g D (dx, dy), D real if REAL.
+template <bool REAL, typename R>
+__device__ __forceinline__ void lc_sub_d(LCCur<R> &acc, R gx, R gy, const Cx<R> &D) {
+  acc.x.re = fma(gx, D.re, acc.x.re);
+  acc.y.re = fma(gy, D.re, acc.y.re);
+  if constexpr (!REAL) {
+    acc.x.im = fma(gx, D.im, acc.x.im);
+    acc.y.im = fma(gy, D.im, acc.y.im);
+  }
+}
+
 // t of the last current for the helicity signs s[a] of the colour positions
 // and s0 of leg 0: |m|^2 = |t|^2 / 2^(L+1) (paper normalisation; the factors
-// 1 / sqrt2 of the polarisation vectors).
+// 1 / sqrt2 of the polarisation vectors).  Products of two legs, and the scalars
+// of two-leg sets, are real.
 template <typename R, int L>
 __device__ __forceinline__ Cx<R> lc_amplitude(const LCOrder<R, L> &o, const R (&s)[L], R s0) {
   LCCur<R> J[L][L];
@@ -166,7 +188,21 @@ __device__ __forceinline__ Cx<R> lc_amplitude(const LCOrder<R, L> &o, const R (&
     return lc_dot(J[a][b], J[c][d]);
   };
 #pragma unroll
-  for (int len = 2; len < L; ++len) {
+  for (int a = 0; a + 1 < L; ++a) {  // two legs: c_r and c_l added up by hand
+    const int b = a + 1;
+    const R pl = o.p[a][a], pr = o.p[b][b], ip = o.ip[a][b], ik = o.ik2[a][b];
+    const R dx = o.bx[a][a] - o.bx[b][b], dy = o.by[a][a] - o.by[b][b];
+    const R ss = s[a] * s[b], D = R(1) - ss, g = (pl * pr) * ip * D, p2 = R(2) * o.p[a][b];
+    const R same = p2 * ss;
+    J[a][b].x = {(fma(R(-2), g, p2) * dx) * ik, (R(2) * fma(pr, s[a], pl * s[b]) * dy) * ik};
+    J[a][b].y = {(fma(R(-2), g, -same) * dy) * ik, (R(2) * fma(pr, s[b], pl * s[a]) * dx) * ik};
+    const R w = (pl - pr) * D * ip;
+    A[a][b] = {D + w, R(0)};
+    B[a][b] = {D - w, R(0)};
+    om[a][b] = {w * ip, R(0)};
+  }
+#pragma unroll
+  for (int len = 3; len < L; ++len) {
 #pragma unroll
     for (int a = 0; a + len - 1 < L; ++a) {
       const int b = a + len - 1;
@@ -175,6 +211,7 @@ __device__ __forceinline__ Cx<R> lc_amplitude(const LCOrder<R, L> &o, const R (&
 #pragma unroll
       for (int i = a; i < b; ++i) {
         const bool ll = i == a, lr = i + 1 == b;
+        const bool l2 = i == a + 1, r2 = i + 2 == b;  // two-leg parts: real scalars
         const R pl = o.p[a][i], pr = o.p[i + 1][b];
         const R dx = o.bx[a][i] - o.bx[i + 1][b], dy = o.by[a][i] - o.by[i + 1][b];
         const Cx<R> D = dot(a, i, i + 1, b);
@@ -184,14 +221,16 @@ __device__ __forceinline__ Cx<R> lc_amplitude(const LCOrder<R, L> &o, const R (&
         } else {
           const LCCur<R> &l = J[a][i];
           cr = {fma(R(2) * pr, fma(l.x.re, dx, fma(l.y.re, dy, om[a][i].re)), A[a][i].re),
-                fma(R(2) * pr, fma(l.x.im, dx, fma(l.y.im, dy, om[a][i].im)), A[a][i].im)};
+                l2 ? (R(2) * pr) * fma(l.x.im, dx, l.y.im * dy)
+                   : fma(R(2) * pr, fma(l.x.im, dx, fma(l.y.im, dy, om[a][i].im)), A[a][i].im)};
         }
         if (lr) {
           cl = {(R(2) * pl) * dx, (R(2) * pl) * (s[b] * dy)};
         } else {
           const LCCur<R> &r = J[i + 1][b];
           cl = {fma(R(2) * pl, fma(r.x.re, dx, fma(r.y.re, dy, -om[i + 1][b].re)), B[i + 1][b].re),
-                fma(R(2) * pl, fma(r.x.im, dx, fma(r.y.im, dy, -om[i + 1][b].im)), B[i + 1][b].im)};
+                r2 ? (R(2) * pl) * fma(r.x.im, dx, r.y.im * dy)
+                   : fma(R(2) * pl, fma(r.x.im, dx, fma(r.y.im, dy, -om[i + 1][b].im)), B[i + 1][b].im)};
         }
         if (lr)
           lc_axpy_leaf(acc, cr, s[b]);
@@ -201,11 +240,8 @@ __device__ __forceinline__ Cx<R> lc_amplitude(const LCOrder<R, L> &o, const R (&
           lc_axpy_leaf(acc, cl, s[a]);
         else
           lc_axpy(acc, cl, J[a][i]);
-        const R gp = R(-2) * (pl * pr) * o.ip[a][b], gx = gp * dx, gy = gp * dy;
-        acc.x.re = fma(gx, D.re, acc.x.re);
-        acc.x.im = fma(gx, D.im, acc.x.im);
-        acc.y.re = fma(gy, D.re, acc.y.re);
-        acc.y.im = fma(gy, D.im, acc.y.im);
+        const R gp = R(-2) * (pl * pr) * o.ip[a][b];
+        lc_sub_d<false>(acc, gp * dx, gp * dy, D);
         S.re += D.re;
         S.im += D.im;
         const R dp = pl - pr;
@@ -217,10 +253,14 @@ __device__ __forceinline__ Cx<R> lc_amplitude(const LCOrder<R, L> &o, const R (&
 #pragma unroll
         for (int j = i + 1; j < b; ++j) {
           const Cx<R> x = dot(a, i, j + 1, b);
-          if (j == i + 1)
-            lc_axpy_leaf(tri, x, s[j]);
-          else
+          if (j > i + 1) {
             lc_axpy(tri, x, J[i + 1][j]);
+          } else if (i == a && j + 1 == b) {  // three legs: x is real
+            tri.x.re += x.re;
+            tri.y.im = fma(s[j], x.re, tri.y.im);
+          } else {
+            lc_axpy_leaf(tri, x, s[j]);
+          }
         }
       }
       const R ik = o.ik2[a][b], ip = o.ip[a][b];
@@ -239,21 +279,28 @@ __device__ __forceinline__ Cx<R> lc_amplitude(const LCOrder<R, L> &o, const R (&
   };
   constexpr int e = L - 1;
   Cx<R> t = zero, tri = zero;
-  auto madd = [](Cx<R> &z, const Cx<R> &u, const Cx<R> &v) {
-    z.re = fma(u.re, v.re, fma(-u.im, v.im, z.re));
-    z.im = fma(u.re, v.im, fma(u.im, v.re, z.im));
+  // z += u v with ru / rv (constants after unrolling): u / v is real
+  auto madd = [](Cx<R> &z, const Cx<R> &u, bool ru, const Cx<R> &v, bool rv) {
+    if (ru && rv)
+      lc_madd<true, true>(z, u, v);
+    else if (ru)
+      lc_madd<true, false>(z, u, v);
+    else if (rv)
+      lc_madd<false, true>(z, u, v);
+    else
+      lc_madd<false, false>(z, u, v);
   };
 #pragma unroll
   for (int i = 0; i < e; ++i) {
-    if (i > 0) madd(t, B[0][i], e0(i + 1, e));
-    if (i + 1 < e) madd(t, A[i + 1][e], e0(0, i));
-    const R kx = R(-2) * o.kx[i], ky = s0 * (R(-2) * o.ky[i]);
-    madd(t, dot(0, i, i + 1, e), Cx<R>{kx, ky});
+    if (i > 0) madd(t, B[0][i], i == 1, e0(i + 1, e), i + 1 == e);
+    if (i + 1 < e) madd(t, A[i + 1][e], i + 2 == e, e0(0, i), i == 0);
+    const Cx<R> k = {R(-2) * o.kx[i], s0 * (R(-2) * o.ky[i])};
+    madd(t, dot(0, i, i + 1, e), i == 0 && i + 1 == e, k, false);
   }
 #pragma unroll
   for (int i = 0; i + 1 < e; ++i)
 #pragma unroll
-    for (int j = i + 1; j < e; ++j) madd(tri, dot(0, i, j + 1, e), e0(i + 1, j));
+    for (int j = i + 1; j < e; ++j) madd(tri, dot(0, i, j + 1, e), i == 0 && j + 1 == e, e0(i + 1, j), i + 1 == j);
   return {fma(R(-2), tri.re, t.re), fma(R(-2), tri.im, t.im)};
 }
 
