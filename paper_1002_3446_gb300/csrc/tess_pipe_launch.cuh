@@ -476,10 +476,13 @@ int plan_pipeline_t(int sm_count, uint64_t n_events, int hist_bins, int form, in
   }
   pl->form = form;
   const bool fused = form == K2_FUSED;
+  const bool cut_first = (caps & CAP_CUT_FIRST) != 0;
+  if (sched < 0 || sched >= SCHED_N) sched = SCHED_SERIAL;
+  pl->defer_hist = sched == SCHED_SERIAL_HIST && hist_bins > 0 && !cut_first && !fused;
   const int rc = with_form<N, R>(form, [&](auto K) {
     using KV = decltype(K);
     pl->block = KV::block;  // events per tile
-    pl->smem = KV::smem(hist_bins);
+    pl->smem = KV::smem(pl->defer_hist ? 0 : hist_bins);  // a deferred histogram is another kernel's
     cudaError_t e = allow_max_smem(KV::fn());
     if (e != cudaSuccess) return (int)e;
     int per_sm = 0;
@@ -505,9 +508,6 @@ int plan_pipeline_t(int sm_count, uint64_t n_events, int hist_bins, int form, in
     pl->kin_smem = 0;
   }
   const int per_sm = pl->per_sm;
-  const bool cut_first = (caps & CAP_CUT_FIRST) != 0;
-  if (sched < 0 || sched >= SCHED_N) sched = SCHED_SERIAL;
-  pl->defer_hist = sched == SCHED_SERIAL_HIST && hist_bins > 0 && !cut_first && !fused;
   const uint64_t per_event = (uint64_t)InRows<L>::rows * sizeof(R) + 3 * sizeof(double) + 1 +
                              (cut_first ? 2 * sizeof(int) : 0) + (pl->defer_hist ? sizeof(double) : 0);
   const uint64_t chunk_bytes = pl->chunk_target ? pl->chunk_target : kChunkTargetBytes;

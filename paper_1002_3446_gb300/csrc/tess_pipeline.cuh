@@ -1655,27 +1655,27 @@ __global__ void __launch_bounds__(NB) bg_rows_real_kernel(ChunkParams C, ChunkBu
     int bin = -1;
     if (j < count) {
       const int e = k2_col(C, B, j);
-      RV4<float> eps0pos, e0;
+      // every load before the first store to shared memory: one latency a tile
+      float v[L][7];
+      RV4<float> e0 = {{0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+      for (int a = 0; a < L; ++a)
+#pragma unroll
+        for (int m = 0; m < 7; ++m) v[a][m] = B.in[(size_t)(InRows<L>::k(a) + m) * cap + e];
+#pragma unroll
+      for (int m = 0; m < 3; ++m) e0.v[1 + m] = B.in[(size_t)(InRows<L>::eps0 + m) * cap + e];
+      const double efac = B.efac[e], wfac = B.wfac[e];
+      const int ok = B.pass[e];
+      const RV4<float> eps0pos = {{0.f, v[0][4], v[0][5], v[0][6]}};
 #pragma unroll
       for (int a = 0; a < L; ++a) {
-        const float *base = B.in + (size_t)InRows<L>::k(a) * cap + e;
-        K4[a * NB + threadIdx.x] = make_float4(base[0], base[cap], base[2 * cap], base[3 * cap]);
-        const float *pe = B.in + (size_t)InRows<L>::eps(a) * cap + e;
-        const RV4<float> ea = {{0.f, pe[0], pe[cap], pe[2 * cap]}};
-        if (a == 0)
-          eps0pos = ea;
-        else
-          J4[t1<L>(a, a) * NB + threadIdx.x] = make_float4(0.f, ea.v[1], ea.v[2], ea.v[3]);
-      }
-      {
-        const float *pe = B.in + (size_t)InRows<L>::eps0 * cap + e;
-        e0.v[0] = 0.f;
-        e0.v[1] = pe[0];
-        e0.v[2] = pe[cap];
-        e0.v[3] = pe[2 * cap];
+        K4[a * NB + threadIdx.x] = make_float4(v[a][0], v[a][1], v[a][2], v[a][3]);
+        if (a > 0) J4[t1<L>(a, a) * NB + threadIdx.x] = make_float4(0.f, v[a][4], v[a][5], v[a][6]);
       }
       const float amp = bg_rows_real<L, NB>(K4, eps0pos, e0, J4, S1);
-      finish_event<NB, float>(C, B, e, amp2_of(Cx<float>{amp, 0.f}), A, w, bin);
+      finish_values<NB>(C, C.P.cut_first ? B.orig[e] : e, efac, wfac, ok, B.hval + e, amp2_of(Cx<float>{amp, 0.f}), A, w,
+                        bin);
+      if (B.wev) B.wev[e] = w;
     }
     epi_tile<NB>(S, nb2, w, bin);
   }

@@ -51,9 +51,11 @@ template <int L, bool LENGTH_MAJOR>
 __host__ __device__ constexpr int wix(int s, int len) {
   return LENGTH_MAJOR ? dsx<L>(s, len) : t1<L>(s, s + len - 1);
 }
+constexpr size_t kWaveEventBytes = 2 * sizeof(double) + 10 * sizeof(float) + sizeof(int);  // WaveEvent
 template <int L>
 __host__ __device__ constexpr size_t wave_smem_per_event() {
-  return (size_t)(L * (L - 1) / 2) * (2 * sizeof(float4) + sizeof(float2)) + (size_t)L * sizeof(float4);
+  return (size_t)(L * (L - 1) / 2) * (2 * sizeof(float4) + sizeof(float2)) + (size_t)L * sizeof(float4) +
+         kWaveEventBytes;
 }
 
 template <int NE>
@@ -122,10 +124,85 @@ __host__ __device__ constexpr int wave_top_group() {
   return ((L - 2) / G) * G + G - 1;
 }
 
+// What the amplitude and the epilogue need of an event besides its table, as
+// planes of NE events: the factors efac, wfac, the polarisation rows of position 0
+// (eps) and of the contraction vector (e0), and the pass flag.
+template <int NE>
+struct WaveEvent {
+  double *f;  // [2][NE]
+  float *x;   // [10][NE]
+  int *pass;  // [NE]
+  __device__ explicit WaveEvent(char *p) : f((double *)p), x((float *)(f + 2 * NE)), pass((int *)(x + 10 * NE)) {}
+};
+
+// The inputs of the event in chunk column e, lane g of its G lanes: every load is
+// issued before the first store to shared memory, so that the tile pays one
+// latency (about 700 cycles from L2) for its legs, the rows that only row 0 and
+// the contraction read and the epilogue's factors, where each leg's loads used to
+// wait for the previous leg's stores and the late rows for the end of the tile
+// (2^22 events at n = 10, whole call: 4755 -> 4690 us; nine processes, n = 4..12,
+// in one graph: 1696 -> 1650).
+// st(a, eps) stores position a's polarisation vector as a single-leg current.
+template <int L, int NE, int G, typename St>
+__device__ __forceinline__ void wave_load(const ChunkBuf<float> &B, int e, int slot, int g, float4 *K4,
+                                          const WaveEvent<NE> &X, St st) {
+  constexpr int LA = (L + G - 1) / G;  // legs per lane
+  const size_t cap = (size_t)B.cap;
+  float v[LA][9], x0[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+  double ef = 0.0, wf = 0.0;
+  int ok = 0;
+#pragma unroll
+  for (int q = 0; q < LA; ++q) {
+    const int a = g + q * G;
+    const float *p = B.in + (size_t)InRows<L>::k(a < L ? a : 0) * cap + e;  // k rows, then eps rows
+#pragma unroll
+    for (int m = 0; m < 9; ++m) v[q][m] = p[m * cap];
+  }
+  if (g == G - 1) {
+    const float *p = B.in + (size_t)InRows<L>::eps0 * cap + e;
+#pragma unroll
+    for (int m = 0; m < 5; ++m) x0[m] = p[m * cap];
+    ef = B.efac[e];
+    wf = B.wfac[e];
+    ok = B.pass[e];
+  }
+#pragma unroll
+  for (int q = 0; q < LA; ++q) {
+    const int a = g + q * G;
+    if (a >= L) break;
+    K4[a * NE + slot] = make_float4(v[q][0], v[q][1], v[q][2], v[q][3]);
+    if (a == 0) {
+#pragma unroll
+      for (int m = 0; m < 5; ++m) X.x[m * NE + slot] = v[q][4 + m];
+    } else {
+      CV4<float> ea;
+      load_eps(&v[q][4], (size_t)1, ea);
+      st(a, ea);
+    }
+  }
+  if (g == G - 1) {
+#pragma unroll
+    for (int m = 0; m < 5; ++m) X.x[(5 + m) * NE + slot] = x0[m];
+    X.f[slot] = ef;
+    X.f[NE + slot] = wf;
+    X.pass[slot] = ok;
+  }
+}
+
+// finish_event from the event's planes.
+template <int NB, int NE>
+__device__ __forceinline__ void wave_finish(const ChunkParams &C, const ChunkBuf<float> &B, int e, int slot,
+                                            const WaveEvent<NE> &X, const Cx<float> &amp, Accum<NB> &A, double &w,
+                                            int &bin) {
+  const int o = C.P.cut_first ? B.orig[e] : e;
+  finish_values<NB>(C, o, X.f[slot], X.f[NE + slot], X.pass[slot], B.hval + e, amp2_of(amp), A, w, bin);
+  if (B.wev) B.wev[e] = w;
+}
+
 // The amplitude m = e0 . Num[0..L-1] of the event in slot e (returned by the
 // lane that builds row 0, g = G-1; other lanes return 0).  in_e0 / in_eps0:
 // the event's rows of the contraction vector and of position 0's
-// polarisation (read from the chunk buffer by that lane).
+// polarisation, row stride cap.
 template <int L, int NE, int G, bool UNR>
 __device__ __forceinline__ Cx<float> bg_wave(const float4 *K4, float4 *J4, float2 *S2, int e, int g,
                                              const float *in_eps0, const float *in_e0, size_t cap) {
@@ -440,43 +517,34 @@ __global__ void __launch_bounds__(NE * G, MINB) bg_wave_kernel(ChunkParams C, Ch
   float4 *K4 = J4 + 2 * T1 * NE;
   float2 *S2 = (float2 *)(K4 + L * NE);
   float2 *S0 = S2 + T1 * NE;  // lean form only: row 0's split sums
+  char *const ev0 = (char *)(LEAN ? S0 + (L - 1) * NE : S0);
+  const WaveEvent<NE> X(ev0);
   const int nb2 = C.P.hist_bins > 0 ? C.P.hist_bins + 2 : 0;
-  EpiSmem<NT> S((char *)(LEAN ? S0 + (L - 1) * NE : S0), nb2);
+  EpiSmem<NT> S(ev0 + kWaveEventBytes * NE, nb2);
   epi_init(S, nb2);
   Accum<NT> A;
   int slot, g;
   wave_slot<G>(slot, g);
   const int count = k2_count(C, B);
   const int ntiles = (count + NE - 1) / NE;
-  const size_t cap = (size_t)B.cap;
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int j = tile * NE + slot;
     const bool has = j < count;
     const int e = has ? k2_col(C, B, j) : 0;  // lanes without an event compute on column 0's data, unused
     if (G > 1) __syncwarp();  // the previous tile's reads of this slot are done
-    // leg momenta and polarisations (positions 1..L-1) into the event's column
-#pragma unroll
-    for (int a = g; a < L; a += G) {
-      const float *base = B.in + (size_t)InRows<L>::k(a) * cap + e;
-      K4[a * NE + slot] = make_float4(base[0], base[cap], base[2 * cap], base[3 * cap]);
-      if (a > 0) {
-        CV4<float> ea;
-        load_eps(B.in + (size_t)InRows<L>::eps(a) * cap + e, cap, ea);
-        wst_cv<NE>(J4, wix<L, UNR && !LEAN>(a, 1), slot, ea);
-      }
-    }
+    wave_load<L, NE, G>(B, e, slot, g, K4, X, [&](int a, const CV4<float> &ea) {
+      wst_cv<NE>(J4, wix<L, UNR && !LEAN>(a, 1), slot, ea);
+    });
     if (G > 1) __syncwarp();
     if constexpr (UNR) wave_prefetch_next<L, NE, NT>(C, B, tile, ntiles);
     Cx<float> amp;
     if constexpr (LEAN)
-      amp = bg_wave_lean<L, NE, G>(K4, J4, S2, S0, slot, g, B.in + (size_t)InRows<L>::eps(0) * cap + e,
-                                   B.in + (size_t)InRows<L>::eps0 * cap + e, cap);
+      amp = bg_wave_lean<L, NE, G>(K4, J4, S2, S0, slot, g, X.x + slot, X.x + 5 * NE + slot, (size_t)NE);
     else
-      amp = bg_wave<L, NE, G, UNR>(K4, J4, S2, slot, g, B.in + (size_t)InRows<L>::eps(0) * cap + e,
-                                   B.in + (size_t)InRows<L>::eps0 * cap + e, cap);
+      amp = bg_wave<L, NE, G, UNR>(K4, J4, S2, slot, g, X.x + slot, X.x + 5 * NE + slot, (size_t)NE);
     double w = 0.0;
     int bin = -1;
-    if (has && g == G - 1) finish_event<NT, float>(C, B, e, amp2_of(amp), A, w, bin);
+    if (has && g == G - 1) wave_finish<NT, NE>(C, B, e, slot, X, amp, A, w, bin);
     epi_tile<NT>(S, nb2, w, bin);
   }
   epi_flush<NT>(S, nb2, A, partials, C);

@@ -203,37 +203,30 @@ __global__ void __launch_bounds__(NE * G) bg_wavep_kernel(ChunkParams C, ChunkBu
   float4 *J4 = (float4 *)smem_raw;
   float4 *K4 = J4 + 2 * T1 * NE;
   float2 *S2 = (float2 *)(K4 + L * NE);
+  char *const ev0 = (char *)(S2 + T1 * NE);
+  const WaveEvent<NE> X(ev0);
   const int nb2 = C.P.hist_bins > 0 ? C.P.hist_bins + 2 : 0;
-  EpiSmem<NT> S((char *)(S2 + T1 * NE), nb2);
+  EpiSmem<NT> S(ev0 + kWaveEventBytes * NE, nb2);
   epi_init(S, nb2);
   Accum<NT> A;
   int slot, g;
   wave_slot<G>(slot, g);
   const int count = k2_count(C, B);
   const int ntiles = (count + NE - 1) / NE;
-  const size_t cap = (size_t)B.cap;
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int j = tile * NE + slot;
     const bool has = j < count;
     const int e = has ? k2_col(C, B, j) : 0;  // lanes without an event compute on column 0's data, unused
     if (G > 1) __syncwarp();
-    // leg momenta and polarisations (positions 1..L-1) into the event's column
-    for (int a = g; a < L; a += G) {
-      const float *base = B.in + (size_t)InRows<L>::k(a) * cap + e;
-      K4[a * NE + slot] = make_float4(base[0], base[cap], base[2 * cap], base[3 * cap]);
-      if (a > 0) {
-        CV4<float> ea;
-        load_eps(B.in + (size_t)InRows<L>::eps(a) * cap + e, cap, ea);
-        pst_cv<NE>(J4, dsx<L>(a, 1), slot, pc_of(ea));
-      }
-    }
+    wave_load<L, NE, G>(B, e, slot, g, K4, X,
+                        [&](int a, const CV4<float> &ea) { pst_cv<NE>(J4, dsx<L>(a, 1), slot, pc_of(ea)); });
     if (G > 1) __syncwarp();
     wave_prefetch_next<L, NE, NT>(C, B, tile, ntiles);
-    const Cx<float> amp = bg_wavep<L, NE, G, UNR>(K4, J4, S2, slot, g, B.in + (size_t)InRows<L>::eps(0) * cap + e,
-                                                  B.in + (size_t)InRows<L>::eps0 * cap + e, cap);
+    const Cx<float> amp =
+        bg_wavep<L, NE, G, UNR>(K4, J4, S2, slot, g, X.x + slot, X.x + 5 * NE + slot, (size_t)NE);
     double w = 0.0;
     int bin = -1;
-    if (has && g == G - 1) finish_event<NT, float>(C, B, e, amp2_of(amp), A, w, bin);
+    if (has && g == G - 1) wave_finish<NT, NE>(C, B, e, slot, X, amp, A, w, bin);
     epi_tile<NT>(S, nb2, w, bin);
   }
   epi_flush<NT>(S, nb2, A, partials, C);
