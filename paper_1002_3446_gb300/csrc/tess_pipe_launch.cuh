@@ -249,19 +249,19 @@ constexpr bool k2_valid(int f, unsigned caps) {
 //   helicity vectors   n = 4  FUSED 111 (REG_TMA_HI 115); 1,000 events 16.5 (20.8,
 //                      it saves a launch), n = 5 160 (REG_HI_PF 157; 17.8, 21.5),
 //                      n = 6 225 (REG_HI 225; 19.8, 25.0)
-//                      n = 7  REG 330 (REG_TMA 332), n = 8 REG 514 (WAVE2U 687, ROWS32 772)
-//                      n = 9  WAVE2U 883 (WAVE2PU 1059, ROWS32 1519), n = 10 1191
-//                      (1450, 1915), n = 11 2282 (2462, 3900)
-//                      n = 12 WAVE2PU 3445 (LANES8 3981, ROWS32 8996)
+//                      n = 7  REG 330 (REG_TMA 332), n = 8 REG 507 (WAVE2U 587, ROWS32 772)
+//                      n = 9  WAVE2U 802 (WAVE2PU 946, ROWS32 1519), n = 10 1091
+//                      (1316, 1915), n = 11 2105 (2242, 3900)
+//                      n = 12 WAVE2PU 2991 (LANES8 3980, ROWS32 8996)
 //   real vectors       n <= 7 REAL_HI 119 / 156 / 201 / 261 (REG 125 / 177 / 258 / 351),
-//                      n = 8, 9 REAL 341 / 447 (ROWS_REAL 364 / 496, ROWS32 792 / 1546)
-//                      n >= 10 ROWS_REAL 771 / 1024 / 1548 (ROWS32 1950 / 3914 / 9036)
+//                      n = 8, 9 REAL 337 / 442 (ROWS_REAL 363 / 496, ROWS32 792 / 1546)
+//                      n >= 10 ROWS_REAL 747 / 1026 / 1537 (ROWS32 1950 / 3914 / 9036)
 // An event's result must not depend on the size of the call it is part of, so the
 // choice follows the number of events only between FUSED and REG_HI, which give the
 // same bits: without a histogram FUSED loses from 2^22 events (n = 4 / 5 / 6: 380 /
 // 578 / 841 us, REG_HI 372 / 534 / 791), with one it does not (391 / 586 / 855, REG_HI
-// 437 / 596 / 863).  (At 1,000 events and n = 8 / 10 / 12 LANES16 would take 30 / 36 / 40
-// us, the choice below 31 / 42 / 59, ROWS32 35 / 56 / 103.)
+// 437 / 596 / 863).  (At 1,000 events and n = 8 / 10 / 12 LANES16 would take 27 / 31 / 38
+// us, the choice below 36 / 41 / 52, ROWS32 35 / 56 / 103.)
 template <int N, typename R>
 int k2_default(unsigned caps, int sched, uint64_t n_events, int hist_bins) {
   if constexpr (sizeof(R) == 8) return K2_LOOP;

@@ -15,7 +15,8 @@
 // occupies G threads instead of one: G times the resident warps for the same
 // shared memory per event.  Lanes whose row is shorter than the group's
 // longest idle at its last steps (for n = 10 and G = 2 the lanes do 83 % of
-// the thread-steps' work).
+// the thread-steps' work; 90 % in the unrolled form, which shares the longest
+// of these steps between the lanes, wave_last).
 //
 // Within a step the split loop over dp is unrolled with a uniform branch per
 // dp (dp < d), so the row's registers are addressed with compile-time
@@ -199,6 +200,135 @@ __device__ __forceinline__ void wave_finish(const ChunkParams &C, const ChunkBuf
   if (B.wev) B.wev[e] = w;
 }
 
+// The last set of a group's longer row, [a..L-1] with D splits, shared by the
+// event's two lanes (unrolled form): lane 1, which built row a, takes the splits
+// behind its legs dp = D-1, D-3, ... with their triples, lane 0, whose row is
+// complete, those behind D-2, D-4, ..., with row a handed over by shuffles.
+// Alone, lane 1 would spend 8 splits and 28 triples on row 0 at n = 10 (a sixth of
+// the kernel's issue slots) with half of the warp idle; shared it is 4 and 16.
+// 2^22 events at n = 10, whole call: 4690 us with no set shared, 4451 with row 0's,
+// about 4360 with row 2's as well (wave_share2).
+// acc: the lanes' sum of the numerator, if the caller wants it (FULL, with the split
+// sum s); otherwise each lane's own part, for row 0 whose contraction is linear.
+template <int L, int NE, int D, bool FULL>
+__device__ __forceinline__ void wave_last(const float4 *K4, const float4 *J4, const float2 *S2, int e, int g, int a,
+                                          CV4<float> (&row)[L - 1], Cx<float> (&srow)[L - 1],
+                                          RV4<float> (&krow)[L - 1], CV4<float> &acc, Cx<float> &s) {
+  constexpr unsigned all = 0xffffffffu;
+  const int src = (threadIdx.x & 31) | 16;  // the event's lane 1
+  const bool hi = g == 1;
+  auto get = [&](float v) { return __shfl_sync(all, v, src); };
+#pragma unroll
+  for (int l = 0; l < D - 1; ++l) {
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      if (l > 0 || m > 0) row[l].c[m].re = get(row[l].c[m].re);
+      if (l > 0 || m == 1 || m == 2) row[l].c[m].im = get(row[l].c[m].im);
+    }
+  }
+  const float4 *const Ja = J4 + 2 * a * NE + e;  // index wix(a + i, len) is a + wix(i, len)
+  // a middle part's first plane: length-major index of length len for lane 1, of
+  // len - 1 for lane 0, whose last leg is one lower
+  const float4 *mid[D];
+#pragma unroll
+  for (int len = 1; len < D; ++len) mid[len] = Ja - (hi ? 0 : 2 * (L - len + 1) * NE);
+  CV4<float> tri = cv_zero<float>();
+  acc = cv_zero<float>();
+  s = cx<float>(0.f, 0.f);
+  RV4<float> kr = {{0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+  for (int dp = D - 1; dp >= 0; dp -= 2) {  // lane 1: dp, lane 0: dp - 1
+    const bool both = dp > 0;
+    kr = radd(kr, wld_k<NE>(K4, a + dp + 1, e));
+    RV4<float> k = kr, kl = krow[dp];
+    CV4<float> Jl = row[dp];
+    Cx<float> sl = srow[dp];
+    if (both) {
+      kr = radd(kr, wld_k<NE>(K4, a + dp, e));
+      const int lo = dp - 1;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const float t = get(krow[lo].v[m]);
+        kl.v[m] = hi ? kl.v[m] : t;
+        k.v[m] = hi ? k.v[m] : kr.v[m];
+        Jl.c[m].re = hi ? Jl.c[m].re : row[lo].c[m].re;
+        Jl.c[m].im = hi ? Jl.c[m].im : row[lo].c[m].im;
+      }
+      const float tr = lo > 0 ? get(srow[lo].re) : 0.f, ti = lo > 0 ? get(srow[lo].im) : 0.f;
+      sl.re = hi ? sl.re : tr;
+      sl.im = hi ? sl.im : ti;
+    }
+    if (both || hi) {
+      const int tr = hi ? dsx<L>(dp + 1, D - dp) : dsx<L>(dp, D - dp + 1);  // the right part, up to leg L-1
+      const CV4<float> Jr = [&] {
+        const float4 u = Ja[2 * tr * NE], v = Ja[(2 * tr + 1) * NE];
+        CV4<float> j;
+        j.c[0] = cx<float>(u.x, u.y);
+        j.c[1] = cx<float>(u.z, u.w);
+        j.c[2] = cx<float>(v.x, v.y);
+        j.c[3] = cx<float>(v.z, v.w);
+        return j;
+      }();
+      const Cx<float> d0 = mdot(Jl, Jr), jlkr = mdot(Jl, k), krjl = mdot(Jr, kl);
+      const Cx<float> cr = cx<float>(2.f * jlkr.re - sl.re, 2.f * jlkr.im - sl.im);
+      Cx<float> cl = cx<float>(-2.f * krjl.re, -2.f * krjl.im);
+      if (dp < D - 1 || !hi) {  // right part has more than one leg
+        const float2 sr = S2[(a + tr) * NE + e];
+        cl.re -= sr.x;
+        cl.im -= sr.y;
+      }
+      axpy(acc, cr, Jr);
+      axpy(acc, cl, Jl);
+      axpy(acc, d0, rsub(kl, k));
+      if (FULL) {
+        s.re += d0.re;
+        s.im += d0.im;
+      }
+#pragma unroll
+      for (int dpp = 0; dpp < dp; ++dpp) {
+        const int len = dp - dpp;  // lane 1's middle part [a+dpp+1..a+dp]; lane 0's is one shorter
+        if (len > 1 || hi) {
+          const float4 *q = mid[len] + 2 * dsx<L>(dpp + 1, len) * NE;
+          const float4 u = q[0], v = q[NE];
+          CV4<float> JB;
+          JB.c[0] = cx<float>(u.x, u.y);
+          JB.c[1] = cx<float>(u.z, u.w);
+          JB.c[2] = cx<float>(v.x, v.y);
+          JB.c[3] = cx<float>(v.z, v.w);
+          const Cx<float> x = dpp == 0 ? mdot_l<true, false>(row[0], Jr) : mdot(row[dpp], Jr);
+          if (len == 1)
+            axpy_leaf(tri, x, JB);
+          else
+            axpy(tri, x, JB);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    acc.c[m].re = fmaf(2.f, tri.c[m].re, acc.c[m].re);
+    acc.c[m].im = fmaf(2.f, tri.c[m].im, acc.c[m].im);
+    if (FULL) {
+      acc.c[m].re += __shfl_xor_sync(all, acc.c[m].re, 16);
+      acc.c[m].im += __shfl_xor_sync(all, acc.c[m].im, 16);
+    }
+  }
+  if (FULL) {
+    s.re += __shfl_xor_sync(all, s.re, 16);
+    s.im += __shfl_xor_sync(all, s.im, 16);
+  }
+}
+
+// Whether row 2's last set is shared as well, measured with both (us per 2^22
+// events, row 0's alone / row 2's too; neither): n = 8 2282 / 2320 (2367), n = 9 3133 /
+// 3141 (3217), n = 10 4361 / 4255 (4570), n = 11 9529 / 8214 (8978), n = 12 18687 / 19650
+// (19484).  Below, the hand-over costs what the shared work saves; at n = 12 the
+// longer code does.
+template <int L>
+__host__ __device__ constexpr bool wave_share2() {
+  return L == 9 || L == 10;
+}
+
 // The amplitude m = e0 . Num[0..L-1] of the event in slot e (returned by the
 // lane that builds row 0, g = G-1; other lanes return 0).  in_e0 / in_eps0:
 // the event's rows of the contraction vector and of position 0's
@@ -317,7 +447,30 @@ __device__ __forceinline__ Cx<float> bg_wave(const float4 *K4, float4 *J4, float
 #pragma unroll
       for (int d = 1; d < L; ++d) {
         if (d > steps) break;
-        step(d);
+        if (G == 2 && d == L - 1) {  // row 0's last set, contracted
+          CV4<float> acc, e0;
+          Cx<float> s;
+          wave_last<L, NE, L - 1, false>(K4, J4, S2, e, g, 0, row, srow, krow, acc, s);
+          load_eps(in_e0, cap, e0);
+          amp = mdot(e0, acc);
+          amp.re += __shfl_xor_sync(0xffffffffu, amp.re, 16);
+          amp.im += __shfl_xor_sync(0xffffffffu, amp.im, 16);
+        } else if (G == 2 && wave_share2<L>() && d == L - 3 && d == steps) {  // row 2's
+          CV4<float> acc;
+          Cx<float> s;
+          wave_last<L, NE, L - 3, true>(K4, J4, S2, e, g, 2, row, srow, krow, acc, s);
+          if (g == 1) {
+            kcur = radd(kcur, wld_k<NE>(K4, L - 1, e));
+            const float inv = 1.f / mdot(kcur, kcur);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) acc.c[m] = cx<float>(acc.c[m].re * inv, acc.c[m].im * inv);
+            constexpr int t = dsx<L>(2, L - 2);  // [2..L-1]
+            wst_cv<NE>(J4, t, e, acc);
+            S2[t * NE + e] = make_float2(s.re, s.im);
+          }
+          __syncwarp();
+        } else
+          step(d);
       }
     } else {
 #pragma unroll 1
