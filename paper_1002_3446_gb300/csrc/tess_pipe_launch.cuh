@@ -258,10 +258,12 @@ constexpr bool k2_valid(int f, unsigned caps) {
 //                      n >= 10 ROWS_REAL 747 / 1026 / 1537 (ROWS32 1950 / 3914 / 9036)
 // An event's result must not depend on the size of the call it is part of, so the
 // choice follows the number of events only between FUSED and REG_HI, which give the
-// same bits: without a histogram FUSED loses from 2^22 events (n = 4 / 5 / 6: 380 /
-// 578 / 841 us, REG_HI 372 / 534 / 791), with one it does not (391 / 586 / 855, REG_HI
-// 437 / 596 / 863).  (At 1,000 events and n = 8 / 10 / 12 LANES16 would take 27 / 31 / 38
-// us, the choice below 36 / 41 / 52, ROWS32 35 / 56 / 103.)
+// same bits: without a histogram FUSED loses above 2^21 events at n = 4 (2^20 106 us,
+// REG_HI 118; 2^21 198, 201; 2^22 379, 371) and from 2^20 at n = 5 and 6 (2^19 87 / 123,
+// REG_HI 88 / 124; 2^20 155 / 226, 154 / 220; 2^21 296 / 433, 282 / 410), with one (40
+// bins) it does not (2^22 events 389 / 585 / 852, REG_HI 429 / 593 / 863).  (At 1,000
+// events and n = 8 / 10 / 12 LANES16 would take 27 / 31 / 38 us, the choice below
+// 36 / 41 / 52, ROWS32 35 / 56 / 103.)
 template <int N, typename R>
 int k2_default(unsigned caps, int sched, uint64_t n_events, int hist_bins) {
   if constexpr (sizeof(R) == 8) return K2_LOOP;
@@ -269,14 +271,14 @@ int k2_default(unsigned caps, int sched, uint64_t n_events, int hist_bins) {
   if (real_eps) return N <= 7 ? K2_REAL_HI : (N <= 9 ? K2_REAL : K2_ROWS_REAL);
   if (N <= 6) {
     const bool fused = k2_valid<N, R>(K2_FUSED, caps) && sched <= SCHED_SERIAL;
-    return fused && (hist_bins > 0 || n_events <= (1u << 21)) ? K2_FUSED : K2_REG_HI;
+    return fused && (hist_bins > 0 || n_events <= (N == 4 ? 1u << 21 : 1u << 19)) ? K2_FUSED : K2_REG_HI;
   }
   return N <= 8 ? K2_REG : (N <= 11 ? K2_WAVE2U : K2_WAVE2PU);
 }
 
 // The schedule that goes with it: the forms with long unrolled bodies leave the
 // histogram to its own kernel (see SCHED_SERIAL_HIST; 2^20 events with 40 bins at
-// n = 9 / 10 / 11 / 12: 906 / 1215 / 2332 / 3479 us against 1122 / 1630 / - / 3552).
+// n = 9 / 10 / 11 / 12: 819 / 1111 / 2134 / 3011 us against 1047 / 1540 / 2929 / 3128).
 inline int k2_default_sched(int form) {
   return form == K2_WAVE2U || form == K2_WAVE2PU || form == K2_ROWS_REAL ? SCHED_SERIAL_HIST : SCHED_SERIAL;
 }

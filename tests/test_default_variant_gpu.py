@@ -16,8 +16,9 @@ def _plan(ctx, n, prec, mode, N, bins=0, flags=0):
 
 
 @pytest.mark.parametrize("n,prec,mode,N,bins,flags,variant,schedule", [
-    (4, DS, S, 1000, 0, 0, tess.TESS_K2_FUSED, 0), (6, DS, S, 1 << 21, 0, 0, tess.TESS_K2_FUSED, 0),
-    (6, DS, S, (1 << 21) + 1, 0, 0, tess.TESS_K2_REG_HI, 0), (6, DS, S, 1 << 24, 40, 0, tess.TESS_K2_FUSED, 0),
+    (4, DS, S, 1000, 0, 0, tess.TESS_K2_FUSED, 0), (4, DS, S, 1 << 21, 0, 0, tess.TESS_K2_FUSED, 0),
+    (4, DS, S, (1 << 21) + 1, 0, 0, tess.TESS_K2_REG_HI, 0), (6, DS, S, 1 << 19, 0, 0, tess.TESS_K2_FUSED, 0),
+    (6, DS, S, (1 << 19) + 1, 0, 0, tess.TESS_K2_REG_HI, 0), (6, DS, S, 1 << 24, 40, 0, tess.TESS_K2_FUSED, 0),
     (5, F32, S, 1000, 0, 0, tess.TESS_K2_REG_HI, 0), (6, DS, S, 1000, 0, tess.TESS_FLAG_CUT_FIRST, tess.TESS_K2_REG_HI, 0),
     (6, DS, R, 1000, 0, 0, tess.TESS_K2_REAL_HI, 0), (7, DS, S, 1000, 40, 0, tess.TESS_K2_REG, 0),
     (7, F32, R, 1000, 0, 0, tess.TESS_K2_REAL_HI, 0), (8, DS, S, 1000, 40, 0, tess.TESS_K2_REG, 0),
