@@ -840,8 +840,19 @@ __device__ __forceinline__ void kin_ds(const ChunkParams &C, const ChunkBuf<floa
 // CF (cut-first): every thread of a block runs the kinematics (threads past
 // the chunk on its last event, writing nothing) so that all reach the
 // compaction point.
+//
+// Resident blocks asked for (0: the compiler's choice, which aims at occupancy by
+// register steps and misses both ways), times to that choice's: FP64-boost form with
+// four (128 registers) 0.98 at n = 4, 6, 0.97 / 1.00 / 0.94 at 7 / 8 / 9, 0.67 / 0.68 /
+// 0.74 at 10 / 11 / 12 (189 registers and two blocks otherwise; 2^19 events at n = 10
+// 549 -> 370 us), 1.01 at n = 5; FP64 form with three 0.98 at n = 6, 10, 0.99 at 8, 1.00
+// at 4, 5, 7, 9, but 1.05 at 12 (one: 0.99).
+template <int N, typename R>
+constexpr int kin_min_blocks() {
+  return sizeof(R) == 4 ? (N == 5 ? 0 : 4) : (N <= 10 ? 3 : 1);
+}
 template <int N, typename R, bool RP = false, bool CF = false>
-__global__ void __launch_bounds__(kBlock) kin_kernel(ChunkParams C, ChunkBuf<R> B) {
+__global__ void __launch_bounds__(kBlock, (kin_min_blocks<N, R>())) kin_kernel(ChunkParams C, ChunkBuf<R> B) {
   const int e = blockIdx.x * kBlock + threadIdx.x;
   if constexpr (sizeof(R) == 4) {
     extern __shared__ __align__(128) float kin_tile[];
