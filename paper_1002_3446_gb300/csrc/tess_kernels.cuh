@@ -29,23 +29,27 @@ __device__ __forceinline__ int hist_bin(double v, double lo, double inv_w, int n
 
 // Fused event kernel.  Each block walks tiles blockIdx.x, blockIdx.x +
 // gridDim.x, ...; each thread keeps FP64 running sums of its own events; the
-// histogram of a tile is filled deterministically (each bin's thread scans
-// the tile's (bin, w) pairs in order); at the end a fixed-shape tree sum
-// writes the block's partial row.  Results are bit-reproducible for a given
-// grid size.  Resident blocks asked for (0: the compiler's choice): four for the
-// FP32 exact sums (2^16 events at n = 5 239 -> 213 us, n = 4 the same); in FP64 none was
-// faster (three and more 5 % slower at n = 5).
+// histogram of a tile is filled deterministically (each bin's thread adds the
+// tile's events of its bin in order, from a bit mask that the events set); at the end
+// a fixed-shape tree sum writes the block's partial row.  Results are
+// bit-reproducible for a given grid size.  (With each bin's thread scanning all 128
+// (bin, w) pairs, every event cost a pass of the FP64 pipe: the exact sum of 2^20
+// events at n = 4 with 50 bins took 2291 us, now 2027.)  Resident blocks asked for
+// (0: the compiler's choice): four for the FP32 exact sums (2^16 events at n = 5 239 ->
+// 213 us, n = 4 the same); in FP64 none was faster (three and more 5 % slower at n = 5).
 template <int N, typename R, bool SUM>
-__global__ void __launch_bounds__(kBlock, sizeof(R) == 4 && SUM ? 4 : 0) event_kernel(EventParams P, double *__restrict__ partials) {
+__global__ void __launch_bounds__(kBlock, sizeof(R) == 4 && SUM ? 4 : 0) event_kernel(EventParams P,
+                                                                                           double *__restrict__ partials) {
   extern __shared__ double smem[];
   const int nb = P.hist_bins;
   const int nb2 = nb > 0 ? nb + 2 : 0;
   double *hw = smem;                             // [nb2]
   double *hw2 = smem + nb2;                      // [nb2]
   double *stage_w = smem + 2 * nb2;              // [kBlock]
-  int *stage_b = (int *)(stage_w + kBlock);      // [kBlock]
+  uint32_t *mask = (uint32_t *)(stage_w + kBlock);  // [nb2][kBlock / 32] the tile's events of each bin
   __shared__ double red[4][kBlock];
   for (int i = threadIdx.x; i < 2 * nb2; i += kBlock) smem[i] = 0.0;
+  for (int i = threadIdx.x; i < nb2 * (kBlock / 32); i += kBlock) mask[i] = 0u;
   double sw = 0.0, sw2 = 0.0, npass = 0.0, nbad = 0.0;
   const uint64_t ntiles = (P.n_events + kBlock - 1) / kBlock;
   for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -76,13 +80,15 @@ __global__ void __launch_bounds__(kBlock, sizeof(R) == 4 && SUM ? 4 : 0) event_k
     if (nb > 0) {
       __syncthreads();
       stage_w[threadIdx.x] = w;
-      stage_b[threadIdx.x] = bin;
+      if (bin >= 0) atomicOr(&mask[bin * (kBlock / 32) + (threadIdx.x >> 5)], 1u << (threadIdx.x & 31));
       __syncthreads();
       for (int b = threadIdx.x; b < nb2; b += kBlock) {
         double a = 0.0, a2 = 0.0;
-        for (int t = 0; t < kBlock; ++t) {
-          if (stage_b[t] == b) {
-            const double x = stage_w[t];
+        for (int q = 0; q < kBlock / 32; ++q) {
+          uint32_t m = mask[b * (kBlock / 32) + q];
+          mask[b * (kBlock / 32) + q] = 0u;
+          for (; m != 0u; m &= m - 1u) {
+            const double x = stage_w[32 * q + __ffs((int)m) - 1];
             a += x;
             a2 += x * x;
           }

@@ -8,7 +8,7 @@ namespace tess {
 
 inline size_t generate_smem(int hist_bins) {
   const int nb2 = hist_bins > 0 ? hist_bins + 2 : 0;
-  return (size_t)(2 * nb2 + kBlock) * sizeof(double) + (size_t)kBlock * sizeof(int);
+  return (size_t)(2 * nb2 + kBlock) * sizeof(double) + (size_t)nb2 * (kBlock / 32) * sizeof(uint32_t);
 }
 
 template <int N, typename R, bool SUM>
