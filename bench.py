@@ -525,7 +525,7 @@ def run_tess(args):
         ms = time_steps(torch, r64, seed, first, max(1, args.steps // 2), 1, flush)
         extra["fp64"] = {"value": n64 / (statistics.mean(ms) * 1e-3), "events": n64,
                          "ms_per_step": statistics.mean(ms),
-                         "achieved_tflops": tess.bg_flops(n) * n64 / (statistics.mean(ms) * 1e-3) / 1e12,
+                         "achieved_tflops": tess.flops_per_event(n, tess.TESS_K2_LOOP) * n64 / (statistics.mean(ms) * 1e-3) / 1e12,
                          "peak_tflops": peaks["fp64"] if peaks else FP64_PEAK_TFLOPS}
         # the main form's per-event error against the FP64 form on the same events
         rf = tess.Run(ctx, proc, n64, per_event=("weight", "me2", "pass"))

@@ -533,8 +533,8 @@ def bg_flops_leaf(n):
 
 
 def bg_flops_wave_unrolled(n):
-    """bg_flops for TESS_K2_WAVE2U (every step's code unrolled), which also
-    leaves out the zeros of single-leg right and last parts."""
+    """bg_flops for TESS_K2_WAVE2U (every step's code unrolled) and TESS_K2_LOOP,
+    which also leave out the zeros of single-leg right and last parts."""
     return _bg_flops_sparse(n, True, False)
 
 
@@ -590,7 +590,7 @@ def flops_per_event(n, variant, random_pol=False, precision=None):
     # the complex-current forms run on real vectors as on helicity vectors
     if variant in REGISTER_FORMS:
         return bg_flops_leaf(n)
-    if variant == 15:  # TESS_K2_WAVE2U
+    if variant in (3, 15):  # TESS_K2_LOOP (first and last trips of its loops apart), TESS_K2_WAVE2U
         return bg_flops_wave_unrolled(n)
     return bg_flops_wave(n) if variant in WAVE_FORMS else bg_flops(n)
 
