@@ -845,11 +845,11 @@ __device__ __forceinline__ void kin_ds(const ChunkParams &C, const ChunkBuf<floa
 // register steps and misses both ways), times to that choice's: FP64-boost form with
 // four (128 registers) 0.98 at n = 4, 6, 0.97 / 1.00 / 0.94 at 7 / 8 / 9, 0.67 / 0.68 /
 // 0.74 at 10 / 11 / 12 (189 registers and two blocks otherwise; 2^19 events at n = 10
-// 549 -> 370 us), 1.01 at n = 5; FP64 form with three 0.98 at n = 6, 10, 0.99 at 8, 1.00
-// at 4, 5, 7, 9, but 1.05 at 12 (one: 0.99).
+// 549 -> 368 us), 1.01 at n = 5; FP64 form with three 0.98 at n = 6, 0.98 / 0.99 (real
+// vectors / helicities) at 8, 1.00 at 4, 5, 7, but spills above (1.05 at 12).
 template <int N, typename R>
 constexpr int kin_min_blocks() {
-  return sizeof(R) == 4 ? (N == 5 ? 0 : 4) : (N <= 10 ? 3 : 1);
+  return sizeof(R) == 4 ? (N == 5 ? 0 : 4) : (N <= 8 ? 3 : 0);
 }
 template <int N, typename R, bool RP = false, bool CF = false>
 __global__ void __launch_bounds__(kBlock, (kin_min_blocks<N, R>())) kin_kernel(ChunkParams C, ChunkBuf<R> B) {
