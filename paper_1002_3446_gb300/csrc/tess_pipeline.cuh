@@ -411,7 +411,10 @@ __device__ __forceinline__ void scatter_legs(const EventParams &P, uint64_t ev, 
 // order; returns this event's column (-1 when it is not kept, i.e. it fails
 // the cuts or lies past the chunk) and records the block's count.  Failing
 // events get their weight and |m|^2 outputs (0) here, since no amplitude
-// kernel sees them.  Every thread of the block must call it.
+// kernel sees them; so do the passing ones, whose amplitude kernel overwrites
+// them: stores of whole lines pass the link to host memory faster than the failing
+// events' alone (2^21 events at n = 8, all outputs in host memory: this kernel 474 ->
+// 458 us, 188 GB/s of the link's 193).  Every thread of the block must call it.
 template <bool CF>
 __device__ __forceinline__ int cut_first_slot(const EventParams &P, const ChunkBuf<float> &B, bool live, int pass,
                                               uint64_t idx, int *kept = nullptr) {
@@ -432,7 +435,7 @@ __device__ __forceinline__ int cut_first_slot(const EventParams &P, const ChunkB
     }
     if (threadIdx.x == 0) B.tcount[blockIdx.x] = tot;
     if (kept) *kept = tot;
-    if (live && !pass) {
+    if (live) {
       if (P.weight) P.weight[idx] = 0.0;
       if (P.me2) P.me2[idx] = 0.0;
     }
